@@ -131,7 +131,7 @@ class ClockSampler:
 # --------------------------------------------------------------------------------------------
 # algorithmic bytes per launch of the three PDHG kernels
 # --------------------------------------------------------------------------------------------
-def kernel_bytes(pb, precision, line_kernels=False):
+def kernel_bytes(pb, precision, line_kernels=False, fused=False):
     """Array touches per grid point of each kernel at the algorithmic minimum, times the point
     count: k_res reads the unknown, the FP32 base state (defect correction, nonlinear kinds)
     and the right-hand side and writes the row-transformed residual; k_col reads and writes
@@ -139,7 +139,7 @@ def kernel_bytes(pb, precision, line_kernels=False):
     unknown and P."""
     es = 4 if precision == "fp32_dc" else 8
     npts = pb.ncomp * pb.nx * pb.ny * getattr(pb, "nz", 1)
-    if getattr(pb, "nz", 1) > 1 or line_kernels:
+    if getattr(pb, "nz", 1) > 1 or (line_kernels and not fused):
         # 3-D: the residual reads the unknown, base state and rhs and writes W; the five transform
         # passes read and write the array (the last also reads and writes P); the update reads
         # P~, the unknown and the base state and writes the unknown.  2-D grids on the same
@@ -152,11 +152,13 @@ def kernel_bytes(pb, precision, line_kernels=False):
         # preconditioner-only transforms 2 + 2 + 2; update dual, Lap P~, A Lap P~, U = 4 + 2 + 3 + 6
         return {"fch_residual": 9 * es * npts, "precond": 6 * es * npts, "fch_update": 15 * es * npts}
     base = 1 if (precision == "fp32_dc" and pb.kind != "none") else 0
-    # k_updres (fused update): k_upd's touches plus the right-hand side read and the transformed
-    # residual written (the unknown is read and written once for both)
+    # fused update: k_fcol as k_col; k_dual reads Y and P and writes P and P~, k_primal reads P~, the
+    # unknown, the base state and the right-hand side and writes the unknown and the residual's
+    # spectrum; k_primal on U_0 (k_primal_first) as k_res
     # k_small*: the one-launch inner solve reads d, u, r, P and writes d once per launch
     return {"k_res": (3 + base) * es * npts, "k_col": 2 * es * npts, "k_upd": (5 + base) * es * npts,
-            "k_updres": (7 + base) * es * npts, "k_small": 5 * es * npts, "k_small_cluster": 5 * es * npts}
+            "k_primal_first": (3 + base) * es * npts, "k_fcol": 2 * es * npts,
+            "k_dual+k_primal": (9 + base) * es * npts, "k_small": 5 * es * npts, "k_small_cluster": 5 * es * npts}
 
 
 def kernel_names(pb, st):
@@ -165,13 +167,15 @@ def kernel_names(pb, st):
         return ("k_small_cluster" if st["small_solve"] == 2 else "k_small",)
     if pb.kind == "fch":
         return ("fch_residual", "precond", "fch_update")
+    if st.get("fused_update"):
+        return ("k_primal_first", "k_fcol", "k_dual+k_primal")
     if getattr(pb, "nz", 1) > 1 or st.get("line_kernels"):
         return ("k3_res", "k3_lines", "k3_upd")
-    return ("k_res", "k_col", "k_updres" if st.get("fused_update") else "k_upd")
+    return ("k_res", "k_col", "k_upd")
 
 
 # the files that define each profiled kernel: a traffic figure stays valid while they are unchanged
-SWEEP_SOURCES = ("rd_sweep.cuh", "rd_device.cuh", "rd_internal.h", "rd_launch.h", "rd_sweep_col.cu",
+SWEEP_SOURCES = ("rd_band.cuh", "rd_fft.cuh", "rd_band_lines.cu", "rd_sweep.cuh", "rd_device.cuh", "rd_internal.h", "rd_launch.h", "rd_sweep_col.cu",
                  "rd_sweep_f32_lap.cu", "rd_sweep_f32_bih.cu", "rd_sweep_f64_lap.cu", "rd_sweep_f64_bih.cu")
 SOURCES_3D = ("rd_3d.cuh", "rd_3d.cu", "rd_sweep.cuh", "rd_device.cuh", "rd_internal.h", "rd_launch3.h")
 KERNEL_SOURCES = {"k_res": SWEEP_SOURCES, "k_col": SWEEP_SOURCES, "k_upd": SWEEP_SOURCES,
@@ -421,7 +425,7 @@ def run_ours(args, rank, world, local_rank):
 
     # per-kernel roofline from the live CUDA-event samples
     peak, peak_kind = load_peaks()
-    kb = kernel_bytes(pb, args.precision, st.get("line_kernels", 0))
+    kb = kernel_bytes(pb, args.precision, st.get("line_kernels", 0), st.get("fused_update", 0))
     names = kernel_names(pb, st)
     per = {}
     for i, nm in enumerate(names):
@@ -440,9 +444,9 @@ def run_ours(args, rank, world, local_rank):
                 "peak_source": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else "fallback",
                 "traffic": read_traffic(args.workload, dom, shash), "per_kernel": per}
         # the whole PDHG sweep of one iteration (k_res + k_col + k_upd, or with the fused update
-        # k_col + k_updres, k_res running only before the first update): algorithmic bytes of its
-        # kernels over the sum of their average durations
-        it_k = [k for k in ("k_col", "k_updres") if k in per] if "k_updres" in per else list(per)
+        # k_fcol + k_dual + k_primal, k_primal on U_0 running only before the first update):
+        # algorithmic bytes of its kernels over the sum of their average durations
+        it_k = [k for k in per if k != "k_primal_first"]
         if len(it_k) >= 2:
             sb = sum(per[k]["algorithmic_bytes"] for k in it_k)
             su = sum(per[k]["avg_us"] for k in it_k)
@@ -484,7 +488,7 @@ def run_ours(args, rank, world, local_rank):
         sv64 = rd.Solver(pb, precision="fp64", profile=1)
         ms64, its64, _ = timed_steps(sv64, u64, args.fp64_steps, 1)
         st64 = sv64.stats()
-        kb64 = kernel_bytes(pb, "fp64", st64.get("line_kernels", 0))
+        kb64 = kernel_bytes(pb, "fp64", st64.get("line_kernels", 0), st64.get("fused_update", 0))
         per64 = {}
         for i, nm in enumerate(kernel_names(pb, st64)):
             n = st64["kernel_samples"][i]

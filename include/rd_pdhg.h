@@ -184,18 +184,18 @@ typedef struct {
                              time; 0: one looped pass body for every pass                       */
     int autotune;         /* 1: at create, time each sweep kernel over a few PDHG iterations at
                              every tile that fits and keep the fastest per kernel (band rows of
-                             k_res and of k_upd, column width of k_col; ignored when band_rows
+                             k_res and of the update, column width of the column solve; ignored when band_rows
                              or col_width is set); 0 (default): the occupancy-based planner.
                              Timing noise can change the choice between runs, and with it the
                              summation order of the stopping norm (results agree to rounding). */
     int dc_stall_window;  /* DC: the FP32 inner solve also stops (as converged) when its residual
                              has not halved for this many updates (its rounding floor); default
                              8                                                                   */
-    int fused_update;     /* 1 (default): FP32 defect correction (either loop) runs the update
-                             of each iteration fused with the next residual (k_col + k_updres
-                             per iteration; k_res only before the first update) when its block
-                             fits, and with autotune only where it measures faster; 0: never.
-                             Fused and unfused inner iterates differ by FP32 rounding only.     */
+    int fused_update;     /* 1 (default): the update of each iteration runs with the next residual
+                             (column solve, k_dual, k_primal per iteration; k_primal alone before
+                             the first update), in FP32 defect correction and plain FP64, on grids
+                             whose transforms it supports (sides of 16 points and more); 0: never.
+                             Fused and unfused iterates differ by rounding only.                 */
     int small_solve;      /* 1 (default): FP32 defect correction on a 2-D grid small enough that
                              every array of the inner solve fits on chip runs each inner solve as
                              ONE kernel launch, its iterations separated by barriers: one block
@@ -221,16 +221,18 @@ typedef struct {
     long long pdhg_iterations;   /* PDHG updates (FP64 plain or FP32 inner)                     */
     long long residual_passes;   /* FP64 residual evaluations of defect correction              */
     long long host_syncs;        /* device -> host status reads                                 */
-    double kernel_ms[3];         /* profile = 1: summed CUDA-event time of k_res, k_col, k_upd   */
+    double kernel_ms[3];         /* profile = 1: summed CUDA-event time of the residual, the
+                                    transforms, the update (fused: k_primal on U_0, the column
+                                    solve, k_dual + k_primal)                                     */
     long long kernel_samples[3]; /* number of timed launches behind kernel_ms                    */
     int plan_band_rows;          /* rows per CTA of the sweeps chosen at create (planner/autotune) */
     int plan_col_width;          /* columns per CTA of the column transform chosen at create      */
-    int plan_upd_rows;           /* rows per CTA of the update sweep (k_upd) chosen at create    */
-    int fused_update;            /* 1 when the fused update + residual kernel (k_updres) runs      */
+    int plan_upd_rows;           /* rows per CTA of the update sweep (k_upd, k_primal)           */
+    int fused_update;            /* 1 when the fused update runs (rd_opts.fused_update)           */
     int small_solve;             /* inner solves in one launch (rd_opts.small_solve): 1 one block,
                                     2 a cluster of eight blocks, 0 the multi-kernel sweeps        */
-    int line_kernels;            /* 1 when the iteration runs on the line-transform kernels (3-D
-                                    grids; 2-D grids with a side beyond the band / column sweeps) */
+    int line_kernels;            /* 1 on 3-D grids and on 2-D grids with a side beyond 2048 (FP32)
+                                    / 4096 (FP64) points                                          */
 } rd_stats;
 
 typedef struct rd_pdhg rd_pdhg;

@@ -1,0 +1,8 @@
+// k_primal in double for the fourth-order equations (thirteen-point biharmonic).
+#include "rd_band.cuh"
+
+namespace rd {
+RD_PRIMAL_KIND(double, KK_CH_IMPL)
+RD_PRIMAL_KIND(double, KK_CH_SPLIT)
+RD_PRIMAL_KIND(double, KK_NONE_BIH)
+}  // namespace rd

@@ -83,6 +83,25 @@ bool use_pingpong(int fft_buffers, int threads, int smem_inplace, int smem_pp) {
   return fft_buffers == 2 || blocks_per_sm<T>(threads, smem_pp) >= blocks_per_sm<T>(threads, smem_inplace);
 }
 
+// Column width of k_fcol (sides of 16 points and more): 32-byte row segments, wider while a block has
+// less than a warp, narrower where a block does not hold that many lines.  Measured in FP32 (column
+// kernel): 2048^2 x 2 16-byte segments 67 us, 32-byte 55 us, 64-byte (one block per SM) 108 us;
+// 1024^2 16.5, 14.1, 16.2 us; 512^2 and 1024 x 128 are flat from 16 to 64 bytes.  Lines too long or
+// too short for it: `old`, the width planned for k_col.
+template <class T>
+int plan_col_width(int nx, int old, Desc d, LaunchCfg c) {
+  int C = std::min(nx, 32 / (int)sizeof(T));
+  auto plan = [&](int w) {
+    d.col_width = w;
+    plan_band<T>(d, 1, kSmemLimit, c);
+    return c.fast_col != 0;
+  };
+  if (plan(C))
+    while (c.thr_fcol < 32 && C < nx && plan(2 * C)) C *= 2;
+  while (C > 2 && !plan(C)) C /= 2;
+  return plan(C) ? C : old;
+}
+
 // Launch shape for one precision.  Returns false when the grid does not fit.
 template <class T>
 // stage_base: the residual kernel stages the defect-correction base rows (Cahn-Hilliard in FP32).
@@ -143,6 +162,11 @@ bool plan_launch(int nx, int ny, int nc, int H, int transform, int neumann, int 
 
       C = cand;
     }
+    if (transform) {
+      c.transform = transform;
+      d.band_rows = d.upd_rows = 2;
+      C = plan_col_width<T>(nx, C, d, c);
+    }
   }
   int smem_col = lines_smem_bytes<T>(C / 2, ny, 0, taby);
   if (smem_col > kSmemLimit) {
@@ -179,7 +203,22 @@ bool plan_launch(int nx, int ny, int nc, int H, int transform, int neumann, int 
   c.smem_upd = smem_upd;
   c.smem_col = smem_col;
   c.transform = transform;
+  plan_band<T>(d, H, kSmemLimit, c);
   return true;
+}
+
+// The fused update's band height: the planner's, halved until a block of k_primal holds it
+// (unchanged where none does).
+template <class T>
+void plan_upd_rows(int ny, int H, Desc& d, LaunchCfg& c) {
+  const int rows0 = d.upd_rows, n0 = d.nupd;
+  plan_band<T>(d, H, kSmemLimit, c);
+  while (!c.fast_row && c.transform && d.upd_rows > 2 && d.upd_rows % 4 == 0) {
+    d.upd_rows /= 2;
+    d.nupd = (ny + d.upd_rows - 1) / d.upd_rows;
+    plan_band<T>(d, H, kSmemLimit, c);
+  }
+  if (!c.fast_row) d.upd_rows = rows0, d.nupd = n0;
 }
 
 }  // namespace
@@ -189,7 +228,8 @@ void rd::set_last_error(const char* msg) { g_last_error = msg ? msg : ""; }
 struct rd_pdhg {
   int nx = 0, ny = 0, nc = 1;
   int nz = 1;       // 3-D grids: points along z (1 on a 2-D grid)
-  int nd3 = 0;      // 1: a 3-D grid (the rd_3d.cu kernels)
+  int nd3 = 0;      // 1: a 3-D grid, or a 2-D grid on the line kernels (rd_3d.cu)
+  int long2d = 0;   // 1: a 2-D side beyond 2048 (FP32) / 4096 (FP64) points
   int small = 0;    // every FP32 inner solve in one launch (rd_small.cu): 1 one block, 2 a cluster
   double hz = 0;
   size_t npts = 0;  // nc * nx * ny * nz
@@ -218,9 +258,7 @@ struct rd_pdhg {
   float* D32 = nullptr;
   float* P32[2] = {nullptr, nullptr};
   float* WY32 = nullptr;
-  float* WY32b = nullptr;   // fused update: second transform buffer
-  float* halo32 = nullptr;  // fused update: per-band copies of U on the halo rows
-  size_t halo_bytes = 0;
+  void* halo = nullptr;     // fused update: per-band copies of U on the halo rows
   float* mu32[2] = {nullptr, nullptr};
   float* r32 = nullptr;
   float* u32 = nullptr;
@@ -432,7 +470,8 @@ rd_status capture_step_graph(rd_pdhg* h, bool first, cudaGraph_t* out, cudaGraph
     if (h->small) return small_launch(h, st, ev);
     if (h->fch) return fch_iteration(h, st, ev);
     if (h->nd3) return h->dc ? launch_iteration3<float>(dd, sti, st, ev) : launch_iteration3<double>(dd, sti, st, ev);
-    if (h->dc && dd.fused) return launch_fused<float>(dd, sti, h->cfg32, st, ev, first_it);
+    if (dd.fused) return h->dc ? launch_fused<float>(dd, sti, h->cfg32, st, ev, first_it)
+                               : launch_fused<double>(dd, sti, h->cfg64, st, ev, first_it);
     return h->dc ? launch_iteration<float>(dd, sti, h->cfg32, st, ev) : launch_iteration<double>(dd, sti, h->cfg64, st, ev);
   };
   auto abort_capture = [&](cudaStream_t st, const char* what, cudaError_t e) {
@@ -473,10 +512,7 @@ rd_status capture_step_graph(rd_pdhg* h, bool first, cudaGraph_t* out, cudaGraph
   // one inner solve on stream st: iteration 1 (with the profiling events when ev), then the
   // WHILE node on handle c (body captured on stream bs) over graph_k iterations per trip
   auto inner_solve = [&](cudaStream_t st, cudaEvent_t* ev, cudaGraphConditionalHandle c, cudaStream_t bs) -> cudaError_t {
-    cudaError_t r = cudaSuccess;
-    // fused update: the per-band halo copies of U start at U_0 = d = 0
-    if (dd.fused) r = cudaMemsetAsync(h->halo32, 0, h->halo_bytes, st);
-    if (r == cudaSuccess) r = iteration(st, ev, true);
+    cudaError_t r = iteration(st, ev, true);
     if (h->small || r != cudaSuccess) return r;
     if ((r = launch_loop_cond(sti, c, 1u, st)) != cudaSuccess) return r;
     return while_node(st, c, bs, no_handle, [&](cudaStream_t b) {
@@ -540,23 +576,23 @@ rd_status capture_step_graph(rd_pdhg* h, bool first, cudaGraph_t* out, cudaGraph
 }
 
 // RD_LOOP_HOST: one graph of graph_k PDHG iterations (profiling events around the first).  With
-// the fused update a second graph starts each inner solve: it clears the halo copies and its
-// first iteration launches k_res; the profiling events sit in that graph only.
+// the fused update a second graph starts each inner solve: its first iteration launches k_primal
+// on U_0 too; the profiling events sit in that graph only.
 rd_status capture_iter_graph(rd_pdhg* h, bool start, cudaGraph_t* graph, cudaGraphExec_t* exec) {
   const int K = h->opts.graph_k;
   const Desc& dd = h->dc ? h->h_desc[1] : h->h_desc[0];
-  const bool fused = h->dc && dd.fused;
+  const bool fused = dd.fused != 0;
   cudaStream_t cs = h->cap_stream;
   RD_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
-  if (fused && start) e = cudaMemsetAsync(h->halo32, 0, h->halo_bytes, cs);
   for (int k = 0; k < (h->small ? 1 : K) && e == cudaSuccess; ++k) {
     cudaEvent_t* ev = (k == 0 && h->opts.profile && (start || !fused)) ? h->ev : nullptr;
     if (h->small) e = small_launch(h, cs, ev);
     else if (h->fch) e = fch_iteration(h, cs, ev);
     else if (h->nd3) e = h->dc ? launch_iteration3<float>(dd, h->d_state + 1, cs, ev)
                                : launch_iteration3<double>(dd, h->d_state + 0, cs, ev);
-    else if (fused) e = launch_fused<float>(dd, h->d_state + 1, h->cfg32, cs, ev, start && k == 0);
+    else if (fused) e = h->dc ? launch_fused<float>(dd, h->d_state + 1, h->cfg32, cs, ev, start && k == 0)
+                              : launch_fused<double>(dd, h->d_state + 0, h->cfg64, cs, ev, start && k == 0);
     else if (h->dc) e = launch_iteration<float>(dd, h->d_state + 1, h->cfg32, cs, ev);
     else e = launch_iteration<double>(dd, h->d_state + 0, h->cfg64, cs, ev);
   }
@@ -576,13 +612,13 @@ rd_status capture_graphs(rd_pdhg* h) {
   h->kernels_per_iter = h->small ? 1
                     : h->fch ? (lc.transform ? 10 : 7)
                     : h->nd3 ? (lc.transform ? (h->nz > 1 ? 7 : 5) : 2)
-                             : (h->dc && h->h_desc[1].fused ? 2 : (lc.transform ? 3 : 2));
+                             : (lc.transform ? 3 : 2);
   if (h->opts.profile)
     for (int i = 0; i < 4; ++i)
       if (!h->ev[i]) RD_CUDA(cudaEventCreate(&h->ev[i]));
   if (h->opts.solve_loop == RD_LOOP_HOST) {
     RD_TRY(capture_iter_graph(h, false, &h->hgraph, &h->hexec));
-    if (h->dc && h->h_desc[1].fused) RD_TRY(capture_iter_graph(h, true, &h->hgraph1, &h->hexec1));
+    if (h->h_desc[h->dc ? 1 : 0].fused) RD_TRY(capture_iter_graph(h, true, &h->hgraph1, &h->hexec1));
     return RD_OK;
   }
   RD_TRY(capture_step_graph(h, true, &h->graph[0], &h->gexec[0]));
@@ -687,16 +723,63 @@ rd_status validate(const rd_grid* grid, rd_bc bc, rd_operator op, const rd_react
   return RD_OK;
 }
 
+// Bytes of the halo copies of U on every band of `rows` rows.
+size_t halo_bytes(int nx, int ny, int nc, int H, int rows, size_t elem) {
+  return (size_t)((ny + rows - 1) / rows) * nc * 2 * H * nx * elem;
+}
+
+// Copies the tiles of one descriptor to another.
+void share_plan(const Desc& d, Desc& o) {
+  o.band_rows = d.band_rows;
+  o.nbands = d.nbands;
+  o.col_width = d.col_width;
+  o.ncolblk = d.ncolblk;
+  o.upd_rows = d.upd_rows;
+  o.nupd = d.nupd;
+}
+
+// Copies the tiles of the planned descriptor d to the handle's others.
+void share_tiles(rd_pdhg* h, const Desc& d) {
+  for (int i : {0, 2}) {
+    share_plan(d, h->h_desc[i]);
+    if (!h->dc) h->h_desc[i].fft_pp = d.fft_pp;
+  }
+}
+
+// Tiles of a 2-D grid with a side beyond the band sweeps of rd_sweep.cuh, on k_fcol, k_dual and
+// k_primal: two-row bands (one line of 8192 points fills a block), the widest columns that fit up to
+// 32 bytes.  False where they cannot run it.
+template <class T>
+bool plan_long(int nx, int ny, int nc, int H, bool neumann, Desc& d, LaunchCfg& c) {
+  (void)neumann;
+  Desc p = d;
+  LaunchCfg q{};
+  p.band_rows = p.upd_rows = 2;
+  p.nbands = p.nupd = ny / 2;
+  q.transform = 1;
+  for (p.col_width = std::min(nx, 32 / (int)sizeof(T)); p.col_width >= 4; p.col_width /= 2) {
+    plan_band<T>(p, H, kSmemLimit, q);
+    if (q.fast_col && q.fast_row) break;
+  }
+  if (p.col_width < 4) return false;
+  p.ncolblk = nx / p.col_width;
+  q.grid_bands = q.grid_upd = p.nupd;
+  q.grid_cols = nc * p.ncolblk;
+  d = p;
+  c = q;
+  return true;
+}
+
 // opts.autotune: on the handle's own arrays (zeroed, with a solve state that never stops, so that
 // every candidate runs the full sweeps) time each kernel over kTuneIters iterations and keep the
-// fastest tiles per kernel: band rows of k_res and of k_upd (each over 2..16 rows), column width
-// of k_col (over 2..64 columns); the three are independent.  Candidates that the planner rejects
-// or that exceed the device's shared memory are skipped.  The choice is reported in rd_stats
-// (plan_band_rows, plan_upd_rows, plan_col_width).
+// fastest tiles per kernel: band rows of k_res and of k_upd (fused: of k_primal; each over 2..16
+// rows), column width of the column kernel (over 2..64 columns); the three are independent.
+// Candidates that the planner rejects or that exceed the device's shared memory are skipped.  The
+// choice is reported in rd_stats (plan_band_rows, plan_upd_rows, plan_col_width).
 constexpr int kTuneIters = 8;
 
 template <class T>
-rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int usable) {
+rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int usable, bool fused) {
   const int ti = h->dc ? 1 : 0;
   cudaStream_t s = h->stream;
   const size_t n = h->npts;
@@ -712,17 +795,30 @@ rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int us
   run.max_iter = 1 << 30;
   run.thresh = -1.0;  // never met: the sweeps stay active
   State* dst = h->d_state + 2;
+  struct Scratch {  // the halo copies of the lowest bands tried
+    void* p = nullptr;
+    ~Scratch() { if (p) cudaFree(p); }
+  } halo;
+  if (fused && cudaMalloc(&halo.p, halo_bytes(h->nx, h->ny, h->nc, H, 2, sizeof(T))) != cudaSuccess) {
+    cudaGetLastError();
+    return RD_OK;  // no room to measure in: keep the planner's choice
+  }
   // per-kernel time (ms, best of three) of kTuneIters iterations for one plan; false if it failed
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   for (int i = 0; i < 4; ++i) RD_CUDA(cudaEventCreate(&ev[i]));
-  auto time_plan = [&](const Desc& dt, const LaunchCfg& ct, float* kms) -> bool {
+  auto iterate = [&](Desc& dt, const LaunchCfg& ct, cudaEvent_t* e, bool first) {
+    dt.fused = fused;
+    dt.halo = halo.p;
+    return fused ? launch_fused<T>(dt, dst, ct, s, e, first) : launch_iteration<T>(dt, dst, ct, s, e);
+  };
+  auto time_plan = [&](Desc& dt, const LaunchCfg& ct, float* kms) -> bool {
     for (int k = 0; k < 3; ++k) kms[k] = 1e30f;
     for (int rep = 0; rep < 3; ++rep) {
       if (cudaMemcpyAsync(dst, &run, sizeof(State), cudaMemcpyHostToDevice, s) != cudaSuccess) return false;
-      if (launch_iteration<T>(dt, dst, ct, s, nullptr) != cudaSuccess) return false;  // warm-up
+      if (iterate(dt, ct, nullptr, true) != cudaSuccess) return false;  // warm-up
       float acc[3] = {0.f, 0.f, 0.f};
       for (int it = 0; it < kTuneIters; ++it) {
-        if (launch_iteration<T>(dt, dst, ct, s, ev) != cudaSuccess) return false;
+        if (iterate(dt, ct, ev, false) != cudaSuccess) return false;
         if (cudaStreamSynchronize(s) != cudaSuccess) return false;
         for (int k = 0; k < 3; ++k) {
           float t = 0.f;
@@ -734,7 +830,9 @@ rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int us
     }
     return true;
   };
-  auto fits = [&](const LaunchCfg& ct) { return std::max(ct.smem_res, std::max(ct.smem_col, ct.smem_upd)) <= usable; };
+  auto fits = [&](const LaunchCfg& ct) {
+    return std::max(ct.smem_res, std::max(ct.smem_col, ct.smem_upd)) <= usable && (!fused || ct.fast_row);
+  };
   std::string why;
   const Desc& d0 = h->h_desc[ti];
   // band rows: k_res and k_upd timed at each height (column width as planned)
@@ -743,8 +841,8 @@ rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int us
   for (int B = 2; B <= 16 && B <= h->ny; B *= 2) {
     Desc dt = d0;
     LaunchCfg ct{};
-    if (!plan_launch<T>(h->nx, h->ny, h->nc, H, transform, h->bc == RD_BC_NEUMANN, B, d0.col_width, B, stage_base,
-                        h->opts.fft_buffers, h->opts.fft_unrolled, dt, ct, why) ||
+    if (!plan_launch<T>(h->nx, h->ny, h->nc, H, transform, h->bc == RD_BC_NEUMANN, fused ? d0.band_rows : B,
+                        d0.col_width, B, stage_base, h->opts.fft_buffers, h->opts.fft_unrolled, dt, ct, why) ||
         !fits(ct))
       continue;
     float kms[3];
@@ -752,10 +850,10 @@ rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int us
       cudaGetLastError();
       continue;
     }
-    if (kms[0] < best_res) best_res = kms[0], bestB = B;
+    if (kms[0] < best_res) best_res = kms[0], bestB = fused ? d0.band_rows : B;
     if (kms[2] < best_upd) best_upd = kms[2], bestU = B;
   }
-  // column width: k_col timed at each width (band rows as planned)
+  // column width: the column kernel timed at each width (band rows as planned)
   if (transform) {
     for (int Cw = 2; Cw <= 64 && Cw <= h->nx; Cw *= 2) {
       if (h->nx % Cw) continue;
@@ -785,93 +883,19 @@ rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int us
     return RD_OK;  // the combination does not fit: keep the planner's choice
   d = dtn;
   lc = tuned;
-  if (h->dc) {
-    h->h_desc[0].band_rows = d.band_rows;
-    h->h_desc[0].nbands = d.nbands;
-    h->h_desc[0].col_width = d.col_width;
-    h->h_desc[0].ncolblk = d.ncolblk;
-    h->h_desc[0].upd_rows = d.upd_rows;
-    h->h_desc[0].nupd = d.nupd;
-  } else {
-    h->cfgpc = lc;
-    Desc& dp = h->h_desc[2];
-    dp.band_rows = d.band_rows;
-    dp.nbands = d.nbands;
-    dp.col_width = d.col_width;
-    dp.ncolblk = d.ncolblk;
-    dp.upd_rows = d.upd_rows;
-    dp.nupd = d.nupd;
-    dp.fft_pp = d.fft_pp;
-  }
-  RD_CUDA(cudaMemcpy(h->d_desc, h->h_desc, 3 * sizeof(Desc), cudaMemcpyHostToDevice));
+  if (!h->dc) h->cfgpc = lc;
+  share_tiles(h, d);
   return RD_OK;
 }
 
-// Fused update (opts.fused_update, FP32 defect correction, either loop): iterations after the
-// first run k_col + k_updres, which needs a second transform buffer and per-band halo copies of
-// U.  Left off when its block does not fit the device's shared memory, and, with opts.autotune,
-// when a fused iteration is not at least 5% faster than an unfused one on this grid.
-rd_status plan_fused(rd_pdhg* h, int H, int stage_base, int usable) {
-  Desc& d = h->h_desc[1];
-  LaunchCfg& lc = h->cfg32;
-  const int U = d.upd_rows, nc = h->nc, nx = h->nx;
-  const int lines = nc * ((U + 4 * H) / 2);
-  const int smem = table_bytes<float>(nx, true, h->bc == RD_BC_NEUMANN) + lines * padded_len(nx) * (int)sizeof(cx<float>) +
-                   nc * (U + 2 * H) * nx * (int)sizeof(float) * (stage_base ? 2 : 1);
-  if (smem > usable) return RD_OK;
-  RD_TRY(dalloc(h, &h->WY32b, h->npts * sizeof(float)));
-  h->halo_bytes = (size_t)d.nupd * nc * 2 * H * nx * sizeof(float);
-  RD_TRY(dalloc(h, &h->halo32, h->halo_bytes));
-  Desc df = d;
-  df.fused = 1;
-  df.WYb[0] = h->WY32;
-  df.WYb[1] = h->WY32b;
-  df.halo = h->halo32;
-  lc.thr_updres = band_threads<float>(lines, nx);
-  lc.smem_updres = smem;
-  if (h->opts.autotune) {
-    // keep the fused update only if a fused iteration is faster than an unfused one here:
-    // kTuneIters iterations of each on the handle's zeroed arrays, a solve that never stops
-    cudaStream_t s = h->stream;
-    for (void* p : {(void*)h->D32, (void*)h->P32[0], (void*)h->P32[1], (void*)h->WY32, (void*)h->WY32b,
-                    (void*)h->r32, (void*)h->u32})
-      RD_CUDA(cudaMemsetAsync(p, 0, h->npts * sizeof(float), s));
-    RD_CUDA(cudaMemsetAsync(h->halo32, 0, h->halo_bytes, s));
-    State run{};
-    run.status = ST_ACTIVE;
-    run.max_iter = 1 << 30;
-    run.thresh = -1.0;
-    State* dst = h->d_state + 2;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    RD_CUDA(cudaEventCreate(&e0));
-    RD_CUDA(cudaEventCreate(&e1));
-    float t[2] = {1e30f, 1e30f};
-    bool ok = true;
-    for (int rep = 0; rep < 3 && ok; ++rep) {
-      for (int f = 0; f < 2 && ok; ++f) {
-        RD_CUDA(cudaMemcpyAsync(dst, &run, sizeof(State), cudaMemcpyHostToDevice, s));
-        ok = (f ? launch_fused<float>(df, dst, lc, s, nullptr, true) : launch_iteration<float>(d, dst, lc, s, nullptr)) ==
-             cudaSuccess;
-        RD_CUDA(cudaEventRecord(e0, s));
-        for (int k = 0; k < kTuneIters && ok; ++k)
-          ok = (f ? launch_fused<float>(df, dst, lc, s, nullptr, false) : launch_iteration<float>(d, dst, lc, s, nullptr)) ==
-               cudaSuccess;
-        RD_CUDA(cudaEventRecord(e1, s));
-        RD_CUDA(cudaStreamSynchronize(s));
-        float ms = 0.f;
-        RD_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-        t[f] = std::min(t[f], ms);
-      }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (!ok) cudaGetLastError();
-    // stream-launched timing flatters the fused loop by a few percent against the graph loop
-    // (measured): demand a 5% margin
-    if (!ok || t[1] >= 0.95f * t[0]) return RD_OK;
-  }
-  d = df;
-  RD_CUDA(cudaMemcpy(h->d_desc, h->h_desc, 3 * sizeof(Desc), cudaMemcpyHostToDevice));
+// Fused update (opts.fused_update, either precision and loop): an iteration is the column kernel,
+// k_dual and k_primal (rd_band.cuh), which needs per-band halo copies of U.
+template <class T>
+rd_status plan_fused(rd_pdhg* h, int H) {
+  Desc& d = h->h_desc[h->dc ? 1 : 0];
+  RD_TRY(dalloc(h, &h->halo, halo_bytes(h->nx, h->ny, h->nc, H, d.upd_rows, sizeof(T))));
+  d.fused = 1;
+  d.halo = h->halo;
   return RD_OK;
 }
 
@@ -887,6 +911,9 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
   if (long2d && rx->kind != RD_RX_NONE && rx->kind != RD_RX_ALLEN_CAHN && rx->kind != RD_RX_CH_IMPLICIT &&
       rx->kind != RD_RX_CH_SPLIT)
     return fail(RD_ERR_UNSUPPORTED, "2-D sides beyond 2048 (FP32) / 4096 (FP64) points are built for the scalar kinds");
+  h->long2d = long2d;
+  // (FP32 inner solves whose both sides k_fcol and the row kernels transform stay on them: decided
+  // below, once the tiles are planned)
   h->nd3 = grid->ndim == 3 || long2d;
   h->nz = grid->ndim == 3 ? grid->n[2] : 1;
   h->nc = rx->ncomp;
@@ -937,7 +964,11 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
 
   std::string why;
   Desc d64 = base, d32 = base;
-  if (h->nd3) {
+  if (long2d && h->dc && transform && h->opts.fused_update &&
+      plan_long<float>(h->nx, h->ny, h->nc, H, bc == RD_BC_NEUMANN, d32, h->cfg32)) {
+    h->nd3 = 0;
+    share_plan(d32, d64);
+  } else if (h->nd3) {
     // 3-D grids: the rd_3d.cu kernels with their own plan (no band / column tiles, no autotuner,
     // no fused update)
     const char* w3 = nullptr;
@@ -949,17 +980,12 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
   } else if (!plan_launch<double>(h->nx, h->ny, h->nc, H, transform, bc == RD_BC_NEUMANN, h->opts.band_rows, h->opts.col_width,
                            h->opts.upd_rows, 0, h->opts.fft_buffers, h->opts.fft_unrolled, d64, h->cfg64, why))
     if (!h->dc) return fail(RD_ERR_UNSUPPORTED, "FP64 path: " + why);
-  if (h->dc && !h->nd3) {
+  if (h->dc && !h->nd3 && !long2d) {
     // the FP64 kernels of the defect-correction loop only need the band decomposition
     if (!plan_launch<float>(h->nx, h->ny, h->nc, H, transform, bc == RD_BC_NEUMANN, h->opts.band_rows, h->opts.col_width,
                            h->opts.upd_rows, rx->kind == RD_RX_CH_IMPLICIT || rx->kind == RD_RX_CH_SPLIT, h->opts.fft_buffers, h->opts.fft_unrolled, d32, h->cfg32, why))
       return fail(RD_ERR_UNSUPPORTED, "FP32 path: " + why);
-    d64.band_rows = d32.band_rows;
-    d64.nbands = d32.nbands;
-    d64.col_width = d32.col_width;
-    d64.ncolblk = d32.ncolblk;
-    d64.upd_rows = d32.upd_rows;
-    d64.nupd = d32.nupd;
+    share_plan(d32, d64);
   }
 
   const size_t n = h->npts;
@@ -1134,18 +1160,35 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
     RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     RD_CUDA(allow_small(optin));
   }
-  if (h->opts.autotune && !h->fch && !h->nd3 && !h->small && h->opts.band_rows == 0 && h->opts.col_width == 0 && h->opts.upd_rows == 0) {
-    const int stage_base = h->dc && (rx->kind == RD_RX_CH_IMPLICIT || rx->kind == RD_RX_CH_SPLIT);
-    RD_TRY(h->dc ? autotune_plan<float>(h, H, transform, stage_base, usable)
-                 : autotune_plan<double>(h, H, transform, stage_base, usable));
+  if (!h->nd3 && !h->small) {
+    const int ti = h->dc ? 1 : 0;
+    Desc& d = h->h_desc[ti];
+    LaunchCfg& c = h->dc ? h->cfg32 : h->cfg64;
+    const bool may_fuse = h->opts.fused_update && transform && !h->fch;
+    if (may_fuse && !h->long2d) {
+      if (h->opts.upd_rows == 0 && h->opts.band_rows == 0) {
+        if (h->dc) plan_upd_rows<float>(h->ny, H, d, c);
+        else plan_upd_rows<double>(h->ny, H, d, c);
+      }
+    }
+    const bool fused = may_fuse && c.fast_row;
+    int dev = 0, optin = 0;
+    RD_CUDA(cudaGetDevice(&dev));
+    RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    RD_CUDA(h->dc ? allow_band<float>(d, c, optin, fused) : allow_band<double>(d, c, optin, fused));
+    if (!h->dc) h->cfgpc = c;
+    share_tiles(h, d);
+    if (h->opts.autotune && !h->fch && !h->long2d && h->opts.band_rows == 0 && h->opts.col_width == 0 && h->opts.upd_rows == 0) {
+      const int stage_base = h->dc && (rx->kind == RD_RX_CH_IMPLICIT || rx->kind == RD_RX_CH_SPLIT);
+      RD_TRY(h->dc ? autotune_plan<float>(h, H, transform, stage_base, usable, fused)
+                   : autotune_plan<double>(h, H, transform, stage_base, usable, fused));
+    }
+    if (fused) RD_TRY(h->dc ? plan_fused<float>(h, H) : plan_fused<double>(h, H));
+    RD_CUDA(cudaMemcpy(h->d_desc, h->h_desc, 3 * sizeof(Desc), cudaMemcpyHostToDevice));
   }
-  if (h->dc && h->opts.fused_update && transform && !h->nd3 && !h->small) {
-    const int stage_base = rx->kind == RD_RX_CH_IMPLICIT || rx->kind == RD_RX_CH_SPLIT;
-    RD_TRY(plan_fused(h, H, stage_base, usable));
-  }
-  h->stats.fused_update = h->h_desc[1].fused;
+  h->stats.fused_update = h->h_desc[h->dc ? 1 : 0].fused;
   h->stats.small_solve = h->small;
-  h->stats.line_kernels = h->nd3;
+  h->stats.line_kernels = grid->ndim == 3 || h->long2d;
   h->stats.plan_band_rows = h->h_desc[h->dc ? 1 : 0].band_rows;
   h->stats.plan_upd_rows = h->h_desc[h->dc ? 1 : 0].upd_rows;
   h->stats.plan_col_width = h->h_desc[h->dc ? 1 : 0].col_width;
@@ -1209,6 +1252,7 @@ rd_status graph_round(rd_pdhg* h, int which) {
     h->stats.kernel_launches += 4 * R - 2 + (sweeps - R) / h->opts.graph_k + (h->h_desc[1].fused ? R : 0);
   } else {
     h->stats.kernel_launches += sweeps > 0 ? 1 + (sweeps - 1) / h->opts.graph_k : 1;
+    if (h->h_desc[h->dc ? 1 : 0].fused) h->stats.kernel_launches += 1;  // k_primal on U_0
   }
   if (h->opts.profile && sweeps > 0) {
     float ms = 0.f;

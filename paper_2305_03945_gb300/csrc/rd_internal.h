@@ -40,9 +40,9 @@ struct Desc {
   int batched;       // 1: member of a batch (Slot control block, device-side phase machine)
   int fft_pp;        // bit 0 k_res, bit 1 k_col, bit 2 k_upd: transforms ping-pong between two buffers;
                      // bit 3: size-specialised unrolled transform passes (else looped passes)
-  int upd_rows;      // rows per CTA of k_upd / k_updres (0: band_rows); k_res keeps band_rows
+  int upd_rows;      // rows per CTA of k_upd / k_primal (0: band_rows); k_res keeps band_rows
   int nupd;          // ceil(ny / upd_rows)
-  int fused;         // 1: iterations after the first run k_col + k_updres (fused update and residual)
+  int fused;         // 1: an iteration is column solve, k_dual, k_primal (update and next residual)
   double hx2, hy2;   // 1/h_x^2, 1/h_y^2
   double dt, a, b;
   double p[6];
@@ -69,11 +69,9 @@ struct Desc {
   float* f32_p0;     // dual P_0 of the inner solve
   float* f32_r;      // r = F(u) rounded to FP32
   float* f32_u;      // u rounded to FP32
-  // fused update + residual (fused = 1): the transform buffer ping-pongs by update parity
-  // (WYb[(n-1)&1] holds the spectrum of update n, k_updres writes F(U_n) into WYb[n&1]); every
-  // k_updres block keeps U on its own halo rows in `halo` ([band][component][2H][nx]), written
-  // and read by that block only
-  void* WYb[2];
+  // fused update (fused = 1): P[0] is the dual (updated in place), P[1] holds P~; every k_primal
+  // block keeps U on its own halo rows in `halo` ([band][component][2H][nx]), written and read by
+  // that block only
   void* halo;
   // 3-D grids (nz > 1; 0 or 1 on a 2-D grid): arrays [ncomp][nz][ny][nx], seven-point Laplacian
   // (the scheme with a third axis), transforms along x, y and z.  Every 3-D kernel runs blk3

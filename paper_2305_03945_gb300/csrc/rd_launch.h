@@ -15,7 +15,13 @@ struct LaunchCfg {
   int smem_res, smem_col, smem_upd;
   int transform;     // 0 when G = I (no spectral solve)
   int grid_upd;      // k_upd bands (0: grid_bands)
-  int thr_updres, smem_updres;  // fused update + residual kernel (k_updres)
+  // kernels on the register-resident transforms (rd_band.cuh), where the sides allow them
+  int fast_col;      // k_fcol in place of k_col
+  int fast_row;      // k_rowfwd, k_dual, k_primal
+  int vcol, vrow;    // values of a line per thread (rd_fft.cuh): 16 or 4
+  int thr_fcol, smem_fcol;
+  int thr_dual, smem_dual;      // k_rowfwd, k_dual
+  int thr_primal, smem_primal;
 };
 
 // Equation keys of the sweep templates (kind_key maps a Desc to one).
@@ -25,23 +31,37 @@ enum KKey {
 };
 
 // Per-key pieces of the sweep, specialised for every (T, K) in the rd_sweep_*.cu units (one unit
-// per group of keys, so that the kernels compile in parallel): one iteration, a k_res launch, and
+// per group of keys, so that the kernels compile in parallel): one iteration and
 // the shared-memory limits of k_res and k_upd.
 template <class T, int K>
 cudaError_t launch_iter_kind(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, cudaEvent_t* ev);
 template <class T, int K>
-cudaError_t launch_res(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s);
-template <class T, int K>
 cudaError_t allow_kind(int optin);
-// The fused FP32 iteration of key K and the shared-memory limit of its k_updres (rd_fused_*.cu).
-template <int K>
-cudaError_t launch_fused_kind(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, cudaEvent_t* ev,
-                              bool first);
-template <int K>
-cudaError_t allow_fused_kind(int optin);
-// The column-transform kernel k_col (pc: the preconditioner-only variant), rd_sweep_col.cu.
+// The column-transform kernel (pc: the preconditioner-only variant), rd_sweep_col.cu: k_fcol where
+// the plan allows it, else k_col.
 template <class T>
 cudaError_t launch_col(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc);
+
+// The kernels of rd_band.cuh: launchers (rd_band_*.cu), the shared-memory limits of the ones the
+// plan (d, c) launches, and the planning rule of their launch shapes.
+template <class T>
+cudaError_t launch_fcol(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc);
+template <class T>
+cudaError_t launch_rowfwd(const Desc& d, const LaunchCfg& c, cudaStream_t s);
+template <class T>
+cudaError_t launch_dual(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc);
+template <class T, int K>
+cudaError_t launch_primal_kind(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool first);
+template <class T, int K>
+cudaError_t allow_primal_kind(const Desc& d, const LaunchCfg& c, int optin);
+template <class T>
+cudaError_t allow_band(const Desc& d, const LaunchCfg& c, int optin, bool primal);
+// threads of a block of these kernels at most, for the element size and values per thread
+inline int band_threads_max(int elem, int vals) { return elem == 8 && vals == 16 ? 256 : 512; }
+// Fills the fast_* part of c for the tiles of d (col_width, upd_rows) and the equation's halo H;
+// col / row: whether k_fcol / the row kernels can run those tiles.
+template <class T>
+void plan_band(const Desc& d, int H, int smem_limit, LaunchCfg& c);
 
 // Raise the dynamic shared-memory limit of the PDHG kernels; *usable receives the bytes a launch may ask.
 template <class T> cudaError_t set_kernel_smem_limits(int* usable);
@@ -49,8 +69,9 @@ template <class T> cudaError_t set_kernel_smem_limits(int* usable);
 // kernels); with ev != NULL, events ev[0..3] are recorded around the three kernels.
 template <class T>
 cudaError_t launch_iteration(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, cudaEvent_t* ev);
-// One PDHG iteration with the fused update (d.fused = 1, FP32 only): k_res (first only), k_col,
-// k_updres; events ev[0..3] around them as in launch_iteration.
+// One PDHG iteration with the fused update (d.fused = 1): k_primal on U_0 (first only), the column
+// kernel, k_dual and k_primal; events ev[0..3] around the three groups (k_dual and k_primal
+// together).
 template <class T>
 cudaError_t launch_fused(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, cudaEvent_t* ev, bool first);
 
