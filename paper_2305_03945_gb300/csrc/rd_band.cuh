@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(BandThreads<T, V>::value) k_dual(const __grid_
   if (!PC && !sweep_active(st, nullptr)) return;
   constexpr int N = F::N;
   const int lline = threadIdx.x / F::TPL, t = threadIdx.x % F::TPL;
-  const int lines = d.ncomp * (d.ny >> 1);
+  const int lines = d.ncomp * (d.ny >> 1) * (d.nz > 1 ? d.nz : 1);
   const int gl = blockIdx.x * (blockDim.x / F::TPL) + lline;
   const bool live = gl < lines;
   cx<T>* line = reinterpret_cast<cx<T>*>(smem_raw) + lline * Lay<T, LOGN, V, false>::len;

@@ -230,6 +230,7 @@ struct rd_pdhg {
   int nz = 1;       // 3-D grids: points along z (1 on a 2-D grid)
   int nd3 = 0;      // 1: a 3-D grid, or a 2-D grid on the line kernels (rd_3d.cu)
   int long2d = 0;   // 1: a 2-D side beyond 2048 (FP32) / 4096 (FP64) points
+  Cube3 cube{};     // FP32 3-D grids on the kernels of rd_cube.cuh
   int small = 0;    // every FP32 inner solve in one launch (rd_small.cu): 1 one block, 2 a cluster
   double hz = 0;
   size_t npts = 0;  // nc * nx * ny * nz
@@ -469,6 +470,7 @@ rd_status capture_step_graph(rd_pdhg* h, bool first, cudaGraph_t* out, cudaGraph
   auto iteration = [&](cudaStream_t st, cudaEvent_t* ev, bool first_it) {
     if (h->small) return small_launch(h, st, ev);
     if (h->fch) return fch_iteration(h, st, ev);
+    if (h->cube.on) return launch_cube(dd, h->cube, sti, st, ev);
     if (h->nd3) return h->dc ? launch_iteration3<float>(dd, sti, st, ev) : launch_iteration3<double>(dd, sti, st, ev);
     if (dd.fused) return h->dc ? launch_fused<float>(dd, sti, h->cfg32, st, ev, first_it)
                                : launch_fused<double>(dd, sti, h->cfg64, st, ev, first_it);
@@ -589,6 +591,7 @@ rd_status capture_iter_graph(rd_pdhg* h, bool start, cudaGraph_t* graph, cudaGra
     cudaEvent_t* ev = (k == 0 && h->opts.profile && (start || !fused)) ? h->ev : nullptr;
     if (h->small) e = small_launch(h, cs, ev);
     else if (h->fch) e = fch_iteration(h, cs, ev);
+    else if (h->cube.on) e = launch_cube(dd, h->cube, h->d_state + 1, cs, ev);
     else if (h->nd3) e = h->dc ? launch_iteration3<float>(dd, h->d_state + 1, cs, ev)
                                : launch_iteration3<double>(dd, h->d_state + 0, cs, ev);
     else if (fused) e = h->dc ? launch_fused<float>(dd, h->d_state + 1, h->cfg32, cs, ev, start && k == 0)
@@ -611,6 +614,7 @@ rd_status capture_graphs(rd_pdhg* h) {
   const LaunchCfg& lc = h->dc ? h->cfg32 : h->cfg64;
   h->kernels_per_iter = h->small ? 1
                     : h->fch ? (lc.transform ? 10 : 7)
+                    : h->cube.on ? 6
                     : h->nd3 ? (lc.transform ? (h->nz > 1 ? 7 : 5) : 2)
                              : (lc.transform ? 3 : 2);
   if (h->opts.profile)
@@ -977,6 +981,7 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
     if (h->dc && !plan3(h->nx, h->ny, h->nz, h->nc, 4, bc == RD_BC_NEUMANN, kSmemLimit, d32, &w3))
       return fail(RD_ERR_UNSUPPORTED, std::string("FP32 path: ") + w3);
     h->cfg64.transform = h->cfg32.transform = transform;
+    if (h->dc && transform) plan_cube(d32, kSmemLimit, h->cube);
   } else if (!plan_launch<double>(h->nx, h->ny, h->nc, H, transform, bc == RD_BC_NEUMANN, h->opts.band_rows, h->opts.col_width,
                            h->opts.upd_rows, 0, h->opts.fft_buffers, h->opts.fft_unrolled, d64, h->cfg64, why))
     if (!h->dc) return fail(RD_ERR_UNSUPPORTED, "FP64 path: " + why);
@@ -994,7 +999,7 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
   const int nb = std::max(d64.nbands, d32.nbands);
   // partials: per band (any band height the autotuner may try) or per step-kernel block
   const int nb_any = std::max(nb, h->ny / 2 + 1);
-  const int nb3 = h->nd3 ? std::max(std::max(d64.blk3, d32.blk3), point_blocks(h->nx, h->ny * h->nz)) : 0;
+  const int nb3 = h->nd3 ? std::max(std::max(std::max(d64.blk3, d32.blk3), h->cube.grid[0]), point_blocks(h->nx, h->ny * h->nz)) : 0;
   RD_TRY(dalloc(h, &h->partials,
                 (size_t)2 * std::max(std::max(std::max(nb_any, point_blocks(h->nx, h->ny)), nb3), 1) * sizeof(double)));
   RD_TRY(dalloc(h, &h->d_desc, 3 * sizeof(Desc)));
@@ -1142,6 +1147,7 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
     RD_CUDA(cudaGetDevice(&dev));
     RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     RD_CUDA(h->dc ? allow3<float>(optin) : allow3<double>(optin));
+    if (h->cube.on) RD_CUDA(allow_cube(d32, h->cube, optin));
     RD_CUDA(allow3<double>(optin));  // the preconditioner-only solve of rd_pdhg_apply_precond
   }
   const LaunchCfg& lc = h->dc ? h->cfg32 : h->cfg64;

@@ -26,6 +26,17 @@ cudaError_t launch_resid64_3(const Desc& hd, const Desc* d64, State* outer, Stat
                              const double* rhs, double* w64, float* r32, float* u32, float* z0, float* z1, int decide,
                              double rtol, int max_outer, cudaStream_t s);
 
+// The FP32 iteration of rd_cube.cuh (sides of 16 .. 1024 points): per axis (x, y, z) the values of a
+// line per thread, the lines (x: row pairs; y, z: column pairs) of a block, its threads, shared
+// memory and the grid.  plan_cube leaves `on` 0 where the kernels of rd_3d.cuh run instead.
+struct Cube3 {
+  int on;
+  int v[3], nl[3], thr[3], smem[3], grid[3];
+};
+void plan_cube(const Desc& d, int smem_limit, Cube3& c);
+cudaError_t allow_cube(const Desc& d, const Cube3& c, int optin);
+cudaError_t launch_cube(const Desc& d, const Cube3& c, State* st, cudaStream_t s, cudaEvent_t* ev);
+
 // Launch plan of the 3-D kernels: blocks per instance (about eight points per thread, at most
 // 1024: one transform tile per block at 128^3, which measured 22% faster than one wave of two
 // blocks per SM) and, per axis, the lines per tile of the transform passes (even,
