@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(LOGN > 12 ? 1024 : 512) k3_lines_long(const __
 __global__ void __launch_bounds__(256) k3_begin(const Desc* __restrict__ d64, State* __restrict__ st,
                                                 const double* __restrict__ uk, double* __restrict__ rhs, double tol,
                                                 int tol_kind) {
+  pdl_wait();
   const Desc& d = *d64;
   __shared__ double red[32];
   const size_t N = (size_t)d.nx * d.ny * d.nz;
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(256)
                const double* __restrict__ u, const double* __restrict__ rhs, double* __restrict__ w64,
                float* __restrict__ r32, float* __restrict__ u32, float* __restrict__ z0, float* __restrict__ z1,
                int decide, double rtol, int max_outer) {
+  pdl_wait();
   if (decide && *((volatile const int*)&outer->status) != ST_ACTIVE) return;
   const Desc& d = *d64;
   __shared__ double red[32];
@@ -288,8 +290,7 @@ bool plan3(int nx, int ny, int nz, int nc, int elem_bytes, bool neumann, int sme
 
 cudaError_t launch_begin3(const Desc& hd, const Desc* d64, State* st, const double* uk, double* rhs, double tol,
                           int tol_kind, cudaStream_t s) {
-  k3_begin<<<hd.blk3, 256, 0, s>>>(d64, st, uk, rhs, tol, tol_kind);
-  return cudaGetLastError();
+  return launch_pdl(k3_begin, hd.blk3, 256, 0, s, d64, st, uk, rhs, tol, tol_kind);
 }
 
 cudaError_t launch_resid64_3(const Desc& hd, const Desc* d64, State* outer, State* inner, const double* u,
@@ -297,13 +298,12 @@ cudaError_t launch_resid64_3(const Desc& hd, const Desc* d64, State* outer, Stat
                              double rtol, int max_outer, cudaStream_t s) {
   const int g = hd.blk3;
   switch (kind_key(hd)) {
-    case KK_AC: k3_resid64<KK_AC><<<g, 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_CH_IMPL: k3_resid64<KK_CH_IMPL><<<g, 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_CH_SPLIT: k3_resid64<KK_CH_SPLIT><<<g, 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_NONE_BIH: k3_resid64<KK_NONE_BIH><<<g, 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    default: k3_resid64<KK_NONE_LAP><<<g, 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
+    case KK_AC: return launch_pdl(k3_resid64<KK_AC>, g, 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_CH_IMPL: return launch_pdl(k3_resid64<KK_CH_IMPL>, g, 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_CH_SPLIT: return launch_pdl(k3_resid64<KK_CH_SPLIT>, g, 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_NONE_BIH: return launch_pdl(k3_resid64<KK_NONE_BIH>, g, 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    default: return launch_pdl(k3_resid64<KK_NONE_LAP>, g, 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace rd

@@ -36,17 +36,16 @@ struct Symbol {
 };
 
 // Spectral scaling of a pair of real columns (a, b) with the symbols of their own frequencies, on
-// the paired middle order v (see rf_pair).  mul(k): eigenvalue of the line axis; ma, mb: of the two
-// columns.  Periodic: with A = (Z + conj Z')/2 and iB = (Z - conj Z')/2 the scaled spectrum is
-// sa A + sb iB = (sa + sb)/2 Z + (sa - sb)/2 conj Z', and the symbols are even in k.  Neumann: the
-// DCT-II coefficients, scaled, and back.
-template <class T, int N, int V>
-__device__ __forceinline__ void scale_pairs(cx<T>* v, int t, bool per, const Symbol<T>& sym, const T* __restrict__ mul,
-                                            const cx<T>* __restrict__ dc, T ma, T mb) {
+// the paired middle order v (see rf_pair).  sym(k, sa, sb): the symbols of the two columns at
+// frequency k of the line.  Periodic: with A = (Z + conj Z')/2 and iB = (Z - conj Z')/2 the scaled
+// spectrum is sa A + sb iB = (sa + sb)/2 Z + (sa - sb)/2 conj Z', and the symbols are even in k.
+// Neumann: the DCT-II coefficients, scaled, and back.
+template <class T, int N, int V, class Sym>
+__device__ __forceinline__ void scale_pairs(cx<T>* v, int t, bool per, const Sym& sym, const cx<T>* __restrict__ dc) {
   auto one = [&](int k, cx<T> z, cx<T> zp, cx<T>& o, cx<T>& op) {
+    T sa, sb;
+    sym(k, sa, sb);
     if (per) {
-      const T m = __ldg(mul + k);
-      const T sa = sym(ma + m), sb = sym(mb + m);
       const T sp = T(0.5) * (sa + sb), sm = T(0.5) * (sa - sb);
       o = cx<T>{sp * z.x + sm * zp.x, sp * z.y - sm * zp.y};
       op = cx<T>{sp * zp.x + sm * z.x, sp * zp.y - sm * z.y};
@@ -54,9 +53,10 @@ __device__ __forceinline__ void scale_pairs(cx<T>* v, int t, bool per, const Sym
       const cx<T> w = ldg(dc + k);
       cx<T> h, hp;
       pair_fwd(false, z, zp, w, h, hp);
-      const T m = __ldg(mul + k), mp = __ldg(mul + (k == 0 ? 0 : N - k));
-      h = cx<T>{h.x * sym(ma + m), h.y * sym(mb + m)};
-      hp = k == 0 ? cx<T>{T(0), T(0)} : cx<T>{hp.x * sym(ma + mp), hp.y * sym(mb + mp)};
+      T ta, tb;
+      sym(k == 0 ? 0 : N - k, ta, tb);
+      h = cx<T>{h.x * sa, h.y * sb};
+      hp = k == 0 ? cx<T>{T(0), T(0)} : cx<T>{hp.x * ta, hp.y * tb};
       pair_inv(false, h, hp, w, o, op);
     }
   };
@@ -81,6 +81,42 @@ __device__ __forceinline__ void scale_pairs(cx<T>* v, int t, bool per, const Sym
     v[V - 1] = op;
   }
   rf_unpair<T, V>(v, t);
+}
+
+// The symbols of the columns with eigenvalues ma, mb from the line axis' eigenvalues mul.
+template <class T>
+struct SymMu {
+  Symbol<T> s;
+  const T* __restrict__ mul;
+  T ma, mb;
+  __device__ __forceinline__ void operator()(int k, T& sa, T& sb) const {
+    const T m = __ldg(mul + k);
+    sa = s(ma + m);
+    sb = s(mb + m);
+  }
+};
+// The same from a table (FP64, whose division and polynomial would take a sixth of the kernel's FP64
+// operations): p points at the pair of columns in row 0, rs elements per row.
+template <class T>
+struct SymTab {
+  const T* __restrict__ p;
+  size_t rs;
+  __device__ __forceinline__ void operator()(int k, T& sa, T& sb) const {
+    const cx<T> v = ldg(reinterpret_cast<const cx<T>*>(p + (size_t)k * rs));
+    sa = v.x;
+    sb = v.y;
+  }
+};
+
+// fills the table of one descriptor: [ncomp][ny][nx]
+static __global__ void __launch_bounds__(256) k_symbol(const __grid_constant__ Desc d, double* __restrict__ out) {
+  const size_t plane = (size_t)d.nx * d.ny;
+  for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < plane * d.ncomp; q += (size_t)gridDim.x * blockDim.x) {
+    const int c = q >= plane ? 1 : 0;
+    const size_t r = q - c * plane;
+    out[q] = Symbol<double>(d, c)(static_cast<const double*>(d.mux)[r & (size_t)(d.nx - 1)] +
+                                  static_cast<const double*>(d.muy)[r >> d.lognx]);
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -109,9 +145,13 @@ __device__ __forceinline__ void fcol_body(const Desc& d, int blk, unsigned char*
   }
   auto sync = [] { __syncthreads(); };
   rf_forward<T, LOGN, V, true>(v, buf, nl, tw, t, sync);
-  const T* mux = static_cast<const T*>(d.mux);
-  scale_pairs<T, N, V>(v, t, per, Symbol<T>(d, c), static_cast<const T*>(d.muy), static_cast<const cx<T>*>(d.dcy),
-                    __ldg(mux + col), __ldg(mux + col + 1));
+  const cx<T>* dc = static_cast<const cx<T>*>(d.dcy);
+  if constexpr (sizeof(T) == 8) {
+    scale_pairs<T, N, V>(v, t, per, SymTab<T>{static_cast<const T*>(d.scale) + (size_t)c * nx * N + col, (size_t)nx}, dc);
+  } else {
+    const T* mux = static_cast<const T*>(d.mux);
+    scale_pairs<T, N, V>(v, t, per, SymMu<T>{Symbol<T>(d, c), static_cast<const T*>(d.muy), __ldg(mux + col), __ldg(mux + col + 1)}, dc);
+  }
   rf_inverse<T, LOGN, V, true>(v, buf, nl, tw, t, sync);
 #pragma unroll
   for (int e = 0; e < V; ++e) {
@@ -133,6 +173,7 @@ struct ColThreads { static constexpr int value = LOGN >= 12 && sizeof(T) == 4 ? 
 template <class T, int LOGN, int V, bool PER>
 __global__ void __launch_bounds__(ColThreads<T, LOGN, V>::value) k_fcol(const __grid_constant__ Desc d, State* __restrict__ st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_wait();
   if (st && !sweep_active(st, nullptr)) return;
   fcol_body<T, LOGN, V, PER>(d, blockIdx.x, smem_raw);
 }
@@ -273,6 +314,7 @@ template <class T, int LOGN, int V>
 __global__ void __launch_bounds__(BandThreads<T, V>::value) k_rowfwd(const __grid_constant__ Desc d) {
   using F = Rf<LOGN, V>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_wait();
   constexpr int N = F::N;
   const int lline = threadIdx.x / F::TPL, t = threadIdx.x % F::TPL;
   const int lines = d.ncomp * (d.ny >> 1);
@@ -302,6 +344,7 @@ template <class T, int LOGN, int V, bool PC>
 __global__ void __launch_bounds__(BandThreads<T, V>::value) k_dual(const __grid_constant__ Desc d, State* __restrict__ st) {
   using F = Rf<LOGN, V>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_wait();
   if (!PC && !sweep_active(st, nullptr)) return;
   constexpr int N = F::N;
   const int lline = threadIdx.x / F::TPL, t = threadIdx.x % F::TPL;
@@ -580,6 +623,7 @@ template <class T, int K, int LOGN, int V>
 __global__ void __launch_bounds__(BandThreads<T, V>::value) k_primal(const __grid_constant__ Desc d, State* __restrict__ st,
                                                                  int first) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_wait();
   if (!sweep_active(st, nullptr)) return;
   primal_body<T, K, LOGN, V>(d, st, blockIdx.x, first != 0, smem_raw);
 }
@@ -631,8 +675,8 @@ inline cudaError_t by_len(int logn, int v, Fn f) {
   template <>                                                                                          \
   cudaError_t launch_primal_kind<T, K>(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool first) { \
     return by_len<T>(d.lognx, c.vrow, [&](auto l, auto v) {                                            \
-      k_primal<T, K, decltype(l)::value, decltype(v)::value><<<d.nupd, c.thr_primal, c.smem_primal, s>>>(d, st, first); \
-      return cudaGetLastError();                                                                       \
+      return launch_pdl(k_primal<T, K, decltype(l)::value, decltype(v)::value>, d.nupd, c.thr_primal,  \
+                        c.smem_primal, s, d, st, first ? 1 : 0);                                       \
     });                                                                                                \
   }                                                                                                    \
   template <>                                                                                          \

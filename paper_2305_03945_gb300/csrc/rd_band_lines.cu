@@ -23,12 +23,18 @@ int line_len(int logn, int vals) {
 
 template <class T>
 cudaError_t launch_fcol(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc) {
+  if (sizeof(T) == 8 && !d.scale) return cudaErrorInvalidValue;  // the handle holds no symbol table
   return by_len<T>(d.logny, c.vcol, [&](auto l, auto v) {
     constexpr int L = decltype(l)::value, V = decltype(v)::value;
-    if (d.bc == BC_PERIODIC) k_fcol<T, L, V, true><<<c.grid_cols, c.thr_fcol, c.smem_fcol, s>>>(d, pc ? nullptr : st);
-    else k_fcol<T, L, V, false><<<c.grid_cols, c.thr_fcol, c.smem_fcol, s>>>(d, pc ? nullptr : st);
-    return cudaGetLastError();
+    return launch_pdl(d.bc == BC_PERIODIC ? k_fcol<T, L, V, true> : k_fcol<T, L, V, false>, c.grid_cols, c.thr_fcol,
+                      c.smem_fcol, s, d, pc ? nullptr : st);
   });
+}
+
+cudaError_t launch_symbol(const Desc& d, double* table, cudaStream_t s) {
+  const size_t n = (size_t)d.ncomp * d.nx * d.ny;
+  k_symbol<<<(unsigned)std::min<size_t>((n + 255) / 256, 8 * 152), 256, 0, s>>>(d, table);
+  return cudaGetLastError();
 }
 
 template <class T>
@@ -36,8 +42,7 @@ cudaError_t launch_rowfwd(const Desc& d, const LaunchCfg& c, cudaStream_t s) {
   return by_len<T>(d.lognx, c.vrow, [&](auto l, auto v) {
     constexpr int L = decltype(l)::value, V = decltype(v)::value;
     const int lpb = c.thr_dual / Rf<L, V>::TPL;
-    k_rowfwd<T, L, V><<<(d.ncomp * (d.ny / 2) + lpb - 1) / lpb, c.thr_dual, c.smem_dual, s>>>(d);
-    return cudaGetLastError();
+    return launch_pdl(k_rowfwd<T, L, V>, (d.ncomp * (d.ny / 2) + lpb - 1) / lpb, c.thr_dual, c.smem_dual, s, d);
   });
 }
 
@@ -47,9 +52,7 @@ cudaError_t launch_dual(const Desc& d, State* st, const LaunchCfg& c, cudaStream
     constexpr int L = decltype(l)::value, V = decltype(v)::value;
     const int lpb = c.thr_dual / Rf<L, V>::TPL;
     const int grid = (d.ncomp * (d.ny / 2) + lpb - 1) / lpb;
-    if (pc) k_dual<T, L, V, true><<<grid, c.thr_dual, c.smem_dual, s>>>(d, st);
-    else k_dual<T, L, V, false><<<grid, c.thr_dual, c.smem_dual, s>>>(d, st);
-    return cudaGetLastError();
+    return launch_pdl(pc ? k_dual<T, L, V, true> : k_dual<T, L, V, false>, grid, c.thr_dual, c.smem_dual, s, d, st);
   });
 }
 

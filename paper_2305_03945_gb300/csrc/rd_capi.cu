@@ -207,18 +207,23 @@ bool plan_launch(int nx, int ny, int nc, int H, int transform, int neumann, int 
   return true;
 }
 
-// The fused update's band height: the planner's, halved until a block of k_primal holds it
-// (unchanged where none does).
+// The fused update's band height: the planner's, halved until a block of k_primal holds it (unchanged
+// where none does).  FP64 at V = 16 is bound by its arithmetic, so the halo rows' share counts more than
+// a full wave of blocks: doubled while the grid keeps 128 bands (1024^2, dual and primal: 2 rows 229 us,
+// 4 rows 201 us, 8 rows 192 us).
 template <class T>
 void plan_upd_rows(int ny, int H, Desc& d, LaunchCfg& c) {
   const int rows0 = d.upd_rows, n0 = d.nupd;
-  plan_band<T>(d, H, kSmemLimit, c);
-  while (!c.fast_row && c.transform && d.upd_rows > 2 && d.upd_rows % 4 == 0) {
-    d.upd_rows /= 2;
-    d.nupd = (ny + d.upd_rows - 1) / d.upd_rows;
+  auto plan = [&](int rows) {
+    d.upd_rows = rows;
+    d.nupd = (ny + rows - 1) / rows;
     plan_band<T>(d, H, kSmemLimit, c);
-  }
-  if (!c.fast_row) d.upd_rows = rows0, d.nupd = n0;
+    return c.fast_row != 0;
+  };
+  int rows = rows0;
+  while (!plan(rows) && c.transform && rows > 2 && rows % 4 == 0) rows /= 2;
+  while (sizeof(T) == 8 && c.fast_row && c.vrow == 16 && ny / (2 * rows) >= 128 && plan(2 * rows)) rows *= 2;
+  if (!plan(rows)) d.upd_rows = rows0, d.nupd = n0;
 }
 
 }  // namespace
@@ -259,6 +264,7 @@ struct rd_pdhg {
   float* D32 = nullptr;
   float* P32[2] = {nullptr, nullptr};
   float* WY32 = nullptr;
+  double* sym64 = nullptr;  // FP64 spectral symbol (k_fcol), rewritten by a change of h_t
   void* halo = nullptr;     // fused update: per-band copies of U on the halo rows
   float* mu32[2] = {nullptr, nullptr};
   float* r32 = nullptr;
@@ -613,7 +619,7 @@ rd_status capture_iter_graph(rd_pdhg* h, bool start, cudaGraph_t* graph, cudaGra
 rd_status capture_graphs(rd_pdhg* h) {
   const LaunchCfg& lc = h->dc ? h->cfg32 : h->cfg64;
   h->kernels_per_iter = h->small ? 1
-                    : h->fch ? (lc.transform ? 10 : 7)
+                    : h->fch ? (fch_fused(h->cfgpc) ? 8 : lc.transform ? 10 : 7)
                     : h->cube.on ? 6
                     : h->nd3 ? (lc.transform ? (h->nz > 1 ? 7 : 5) : 2)
                              : (lc.transform ? 3 : 2);
@@ -658,6 +664,7 @@ rd_status set_dt_impl(rd_pdhg* h, double dt) {
     symbol_coefficients(h, h->h_desc[i]);
   }
   RD_CUDA(cudaMemcpy(h->d_desc, h->h_desc, 3 * sizeof(Desc), cudaMemcpyHostToDevice));
+  if (h->sym64) RD_CUDA(launch_symbol(h->h_desc[0], h->sym64, h->stream));
   destroy_graphs(h);
   return capture_graphs(h);
 }
@@ -1181,8 +1188,14 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
     int dev = 0, optin = 0;
     RD_CUDA(cudaGetDevice(&dev));
     RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    if (!h->dc && c.fast_col) {
+      RD_TRY(dalloc(h, &h->sym64, h->npts * sizeof(double)));
+      RD_CUDA(launch_symbol(d, h->sym64, h->stream));
+      h->h_desc[0].scale = h->h_desc[2].scale = h->sym64;
+    }
     RD_CUDA(h->dc ? allow_band<float>(d, c, optin, fused) : allow_band<double>(d, c, optin, fused));
     if (!h->dc) h->cfgpc = c;
+    if (h->fch && fch_fused(h->cfgpc)) RD_CUDA(allow_fch(d, h->cfgpc, optin));
     share_tiles(h, d);
     if (h->opts.autotune && !h->fch && !h->long2d && h->opts.band_rows == 0 && h->opts.col_width == 0 && h->opts.upd_rows == 0) {
       const int stage_base = h->dc && (rx->kind == RD_RX_CH_IMPLICIT || rx->kind == RD_RX_CH_SPLIT);

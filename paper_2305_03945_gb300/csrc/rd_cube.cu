@@ -53,8 +53,8 @@ int line_len3(int logn, int vals) {
 template <int AX, int MODE>
 cudaError_t launch_axis(const Desc& d, const Cube3& c, State* st, cudaStream_t s) {
   return by_len3(AX == 1 ? d.logny : d.lognz, c.v[AX], [&](auto l, auto v) {
-    k3_axis<float, AX, MODE, decltype(l)::value, decltype(v)::value><<<c.grid[AX], c.thr[AX], c.smem[AX], s>>>(d, st, c.nl[AX]);
-    return cudaGetLastError();
+    return launch_pdl(k3_axis<float, AX, MODE, decltype(l)::value, decltype(v)::value>, c.grid[AX], c.thr[AX], c.smem[AX],
+                      s, d, st, c.nl[AX]);
   });
 }
 
@@ -68,8 +68,7 @@ cudaError_t iteration_k(const Desc& d, const Cube3& c, State* st, cudaStream_t s
   mark(0);
   if (e == cudaSuccess)
     e = by_len3(d.lognx, c.v[0], [&](auto l, auto v) {
-      k3_rowres<float, K, decltype(l)::value, decltype(v)::value><<<c.grid[0], c.thr[0], c.smem[0], s>>>(d, st);
-      return cudaGetLastError();
+      return launch_pdl(k3_rowres<float, K, decltype(l)::value, decltype(v)::value>, c.grid[0], c.thr[0], c.smem[0], s, d, st);
     });
   mark(1);
   if (e == cudaSuccess) e = launch_axis<1, L3_FWD>(d, c, st, s);
@@ -77,14 +76,11 @@ cudaError_t iteration_k(const Desc& d, const Cube3& c, State* st, cudaStream_t s
   if (e == cudaSuccess) e = launch_axis<1, L3_INV>(d, c, st, s);
   if (e == cudaSuccess)
     e = by_len3(d.lognx, c.v[0], [&](auto l, auto v) {
-      k_dual<float, decltype(l)::value, decltype(v)::value, false><<<c.grid[0], c.thr[0], c.smem[0], s>>>(d, st);
-      return cudaGetLastError();
+      return launch_pdl(k_dual<float, decltype(l)::value, decltype(v)::value, false>, c.grid[0], c.thr[0], c.smem[0], s, d, st);
     });
   mark(2);
-  if (e == cudaSuccess) {
-    k3_primal<float, K><<<(unsigned)(((size_t)d.nx * d.ny * d.nz / 4 + 255) / 256), 256, 0, s>>>(d, st);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess)
+    e = launch_pdl(k3_primal<float, K>, (unsigned)(((size_t)d.nx * d.ny * d.nz / 4 + 255) / 256), 256, 0, s, d, st);
   mark(3);
   return e;
 }

@@ -129,6 +129,7 @@ __device__ __forceinline__ void rowres3_body(const Desc& d, State* __restrict__ 
 template <class T, int K, int LOGN, int V>
 __global__ void __launch_bounds__(256) k3_rowres(const __grid_constant__ Desc d, State* __restrict__ st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_wait();
   if (!sweep_active(st, nullptr)) return;
   rowres3_body<T, K, LOGN, V>(d, st, nullptr, blockIdx.x, gridDim.x, smem_raw);
 }
@@ -170,8 +171,10 @@ __device__ __forceinline__ void axis3_body(const Desc& d, int nl, int blk, unsig
     const T* mux = static_cast<const T*>(d.mux);
     const T* muo = static_cast<const T*>(AX == 1 ? d.muz : d.muy);
     const T mo = __ldg(muo + third);
-    scale_pairs<T, N, V>(v, t, per, Symbol<T>(d, 0), static_cast<const T*>(AX == 1 ? d.muy : d.muz), dc,
-                         __ldg(mux + 2 * col) + mo, __ldg(mux + 2 * col + 1) + mo);
+    scale_pairs<T, N, V>(v, t, per,
+                         SymMu<T>{Symbol<T>(d, 0), static_cast<const T*>(AX == 1 ? d.muy : d.muz),
+                                  __ldg(mux + 2 * col) + mo, __ldg(mux + 2 * col + 1) + mo},
+                         dc);
   }
   if constexpr (MODE == L3_FWD) {
     rf_pair<T, V>(v, t);
@@ -229,6 +232,7 @@ template <class T, int AX, int MODE, int LOGN, int V>
 __global__ void __launch_bounds__(BandThreads<T, V>::value) k3_axis(const __grid_constant__ Desc d, State* __restrict__ st,
                                                                     int nl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_wait();
   if (st && !sweep_active(st, nullptr)) return;  // st = nullptr: the preconditioner alone
   axis3_body<T, AX, MODE, LOGN, V>(d, nl, blockIdx.x, smem_raw);
 }
@@ -259,6 +263,7 @@ __device__ __forceinline__ void primal3_body(const Desc& d, int blk) {
 
 template <class T, int K>
 __global__ void __launch_bounds__(256) k3_primal(const __grid_constant__ Desc d, State* __restrict__ st) {
+  pdl_wait();
   if (!sweep_active(st, nullptr)) return;
   primal3_body<T, K>(d, blockIdx.x);
 }

@@ -9,6 +9,33 @@
 
 namespace rd {
 
+// Programmatic dependent launch.  A kernel launched with launch_pdl is scheduled once the blocks of
+// the kernel before it have exited, without waiting for that grid's completion to be flushed and
+// reported; pdl_wait(), its first statement, waits until everything the kernels before it wrote is
+// visible.  Every kernel of a chain calls it, whatever it does afterwards: the kernel behind it waits
+// for this one alone.  The kernels give no earlier signal (griddepcontrol.launch_dependents): with it
+// the next grid's blocks settled unevenly on the SMs the last wave had left, and steps got slower
+// (1024 x 128 834 -> 1093 us, 1024^2 752 -> 794 us, FP64 1024^2 4.83 -> 5.27 ms).  Without it: 834 ->
+// 812 us, 512^2 749 -> 730 us, 128^3 1954 -> 1911 us, FP64 preconditioner 128^2 x 2 54 -> 49 us.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 template <class T> struct cx { T x, y; };
 
 template <class T> __device__ __forceinline__ cx<T> cadd(cx<T> a, cx<T> b) { return {a.x + b.x, a.y + b.y}; }

@@ -52,7 +52,8 @@ struct Desc {
   const void* rhs;   // plain: rhs of the step (FP64); DC: r = F(u) rounded to FP32
   void* P[2];        // dual variable, ping-pong by iteration parity
   void* WY;          // transform buffer: F(U) row-transformed, then G^{-1}-scaled spectrum
-  const void* scale; // unused by the sweeps (kept for layout); see mux / muy
+  const void* scale; // FP64: the spectral symbol 1 / (g_hat nx ny), [ncomp][ny][nx] (k_fcol); else formed from
+                     // mux and muy on the fly (nullptr)
   const void* mux;   // nx entries of T: 4/h_x^2 sin^2(pi kx / (d nx)), d = 1 periodic, 2 Neumann
   const void* muy;   // ny entries of T
   double gc1[2];     // per component: g_hat = (1 + gc1 mu + gc2 mu^2 + gc3 mu^3)^2, mu = mux + muy

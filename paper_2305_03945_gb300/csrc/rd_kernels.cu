@@ -39,6 +39,7 @@ __device__ __forceinline__ double2 ld2(const double* p) { return *reinterpret_ca
 __global__ void __launch_bounds__(256) k_begin(const Desc* __restrict__ d64, State* __restrict__ st,
                                                const double* __restrict__ uk, double* __restrict__ rhs, double tol,
                                                int tol_kind) {
+  pdl_wait();
   const Desc& d = *d64;
   __shared__ double red[32];
   const int nx = d.nx, ny = d.ny, nc = d.ncomp, bc = d.bc;
@@ -98,6 +99,7 @@ __global__ void __launch_bounds__(256)
               const double* __restrict__ u, const double* __restrict__ rhs, double* __restrict__ w64,
               float* __restrict__ r32, float* __restrict__ u32, float* __restrict__ z0, float* __restrict__ z1,
               int decide, double rtol, int max_outer) {
+  pdl_wait();
   if (decide && *((volatile const int*)&outer->status) != ST_ACTIVE) return;
   const Desc& d = *d64;
   __shared__ double red[32];
@@ -156,6 +158,7 @@ constexpr unsigned kLoopSlack = 1024;
 // whatever the stopping logic does, when the count exceeds max_iter + kLoopSlack, else to 1.
 // Kept out of the sweep kernels, which thereby use no device-side graph API.
 __global__ void k_loop_cond(State* __restrict__ st, cudaGraphConditionalHandle cond, unsigned sweeps) {
+  pdl_wait();
   volatile State* vs = st;
   const unsigned t = vs->trips + sweeps;
   vs->trips = t;
@@ -170,6 +173,7 @@ __global__ void k_loop_cond(State* __restrict__ st, cudaGraphConditionalHandle c
 // updates and k_res launches to the outer state's totals.  n is a multiple of 4.
 __global__ void k_axpy_dc(double* __restrict__ u, const float* __restrict__ dlt, size_t n, State* __restrict__ outer,
                           const State* __restrict__ inner) {
+  pdl_wait();
   if (*((volatile const int*)&outer->status) != ST_ACTIVE) return;
   const int is = *((volatile const int*)&inner->status);
   const bool ok = is == ST_CONVERGED || is == ST_NOT_CONVERGED;
@@ -196,6 +200,7 @@ __global__ void k_axpy_dc(double* __restrict__ u, const float* __restrict__ dlt,
 // h_x h_y (h_z) sum of u into st->mass; with `gate`, only once `gate` is no longer active.
 __global__ void __launch_bounds__(256) k_mass(const Desc* __restrict__ d64, State* __restrict__ st,
                                               const double* __restrict__ u, const State* __restrict__ gate) {
+  pdl_wait();
   if (gate && *((volatile const int*)&gate->status) == ST_ACTIVE) return;
   const Desc& d = *d64;
   __shared__ double red[32];
@@ -237,38 +242,33 @@ static int wave_blocks(F kernel, int nblocks) {
 
 cudaError_t launch_begin(const Desc* d64, State* st, const double* uk, double* rhs, double tol, int tol_kind,
                          int nblocks, cudaStream_t s) {
-  k_begin<<<wave_blocks(k_begin, nblocks), 256, 0, s>>>(d64, st, uk, rhs, tol, tol_kind);
-  return cudaGetLastError();
+  return launch_pdl(k_begin, wave_blocks(k_begin, nblocks), 256, 0, s, d64, st, uk, rhs, tol, tol_kind);
 }
 
 cudaError_t launch_resid64(const Desc& hd, const Desc* d64, State* outer, State* inner, const double* u,
                            const double* rhs, double* w64, float* r32, float* u32, float* z0, float* z1, int decide,
                            double rtol, int max_outer, int nblocks, cudaStream_t s) {
   switch (kind_key(hd)) {
-    case KK_AC: k_resid64<KK_AC><<<wave_blocks(k_resid64<KK_AC>, nblocks), 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_CH_IMPL: k_resid64<KK_CH_IMPL><<<wave_blocks(k_resid64<KK_CH_IMPL>, nblocks), 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_CH_SPLIT: k_resid64<KK_CH_SPLIT><<<wave_blocks(k_resid64<KK_CH_SPLIT>, nblocks), 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_GS: k_resid64<KK_GS><<<wave_blocks(k_resid64<KK_GS>, nblocks), 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_SCHNAK: k_resid64<KK_SCHNAK><<<wave_blocks(k_resid64<KK_SCHNAK>, nblocks), 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    case KK_NONE_BIH: k_resid64<KK_NONE_BIH><<<wave_blocks(k_resid64<KK_NONE_BIH>, nblocks), 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
-    default: k_resid64<KK_NONE_LAP><<<wave_blocks(k_resid64<KK_NONE_LAP>, nblocks), 256, 0, s>>>(d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer); break;
+    case KK_AC: return launch_pdl(k_resid64<KK_AC>, wave_blocks(k_resid64<KK_AC>, nblocks), 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_CH_IMPL: return launch_pdl(k_resid64<KK_CH_IMPL>, wave_blocks(k_resid64<KK_CH_IMPL>, nblocks), 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_CH_SPLIT: return launch_pdl(k_resid64<KK_CH_SPLIT>, wave_blocks(k_resid64<KK_CH_SPLIT>, nblocks), 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_GS: return launch_pdl(k_resid64<KK_GS>, wave_blocks(k_resid64<KK_GS>, nblocks), 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_SCHNAK: return launch_pdl(k_resid64<KK_SCHNAK>, wave_blocks(k_resid64<KK_SCHNAK>, nblocks), 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    case KK_NONE_BIH: return launch_pdl(k_resid64<KK_NONE_BIH>, wave_blocks(k_resid64<KK_NONE_BIH>, nblocks), 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
+    default: return launch_pdl(k_resid64<KK_NONE_LAP>, wave_blocks(k_resid64<KK_NONE_LAP>, nblocks), 256, 0, s, d64, outer, inner, u, rhs, w64, r32, u32, z0, z1, decide, rtol, max_outer);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_axpy_dc(double* u, const float* dlt, size_t n, State* outer, const State* inner, cudaStream_t s) {
-  k_axpy_dc<<<wave_blocks(k_axpy_dc, (int)((n / 4 + 255) / 256)), 256, 0, s>>>(u, dlt, n, outer, inner);
-  return cudaGetLastError();
+  return launch_pdl(k_axpy_dc, wave_blocks(k_axpy_dc, (int)((n / 4 + 255) / 256)), 256, 0, s, u, dlt, n, outer, inner);
 }
 
 cudaError_t launch_loop_cond(State* st, unsigned long long cond, unsigned sweeps, cudaStream_t s) {
-  k_loop_cond<<<1, 1, 0, s>>>(st, (cudaGraphConditionalHandle)cond, sweeps);
-  return cudaGetLastError();
+  return launch_pdl(k_loop_cond, 1, 1, 0, s, st, (cudaGraphConditionalHandle)cond, sweeps);
 }
 
 cudaError_t launch_mass(const Desc* d64, State* st, const double* u, const State* gate, int nblocks, cudaStream_t s) {
-  k_mass<<<wave_blocks(k_mass, nblocks), 256, 0, s>>>(d64, st, u, gate);
-  return cudaGetLastError();
+  return launch_pdl(k_mass, wave_blocks(k_mass, nblocks), 256, 0, s, d64, st, u, gate);
 }
 
 }  // namespace rd

@@ -46,6 +46,8 @@ cudaError_t launch_col(const Desc& d, State* st, const LaunchCfg& c, cudaStream_
 // plan (d, c) launches, and the planning rule of their launch shapes.
 template <class T>
 cudaError_t launch_fcol(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc);
+// The FP64 symbol table k_fcol<double> reads through Desc::scale ([ncomp][ny][nx]).
+cudaError_t launch_symbol(const Desc& d, double* table, cudaStream_t s);
 template <class T>
 cudaError_t launch_rowfwd(const Desc& d, const LaunchCfg& c, cudaStream_t s);
 template <class T>
@@ -103,6 +105,11 @@ cudaError_t launch_fch_residual(const Desc& d, State* st, const FchBuffers& b, c
 // Events ev[0..3] (may be NULL) around the residual, the preconditioner solve and the update.
 cudaError_t launch_fch_iteration(const Desc& d, const Desc& dpc, State* st, State* st_pc, const LaunchCfg& cpc,
                                  const FchBuffers& b, int max_blocks, cudaStream_t s, cudaEvent_t* ev);
+
+// Whether that iteration runs its fused form (eight launches; else ten with G, seven without), and the
+// shared-memory limit of its kernels.
+bool fch_fused(const LaunchCfg& cpc);
+cudaError_t allow_fch(const Desc& d, const LaunchCfg& cpc, int optin);
 
 // Set the thread-local detail string returned by rd_last_error().
 void set_last_error(const char* msg);
