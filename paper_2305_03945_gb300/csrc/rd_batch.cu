@@ -363,9 +363,9 @@ struct rd_batch {
   int2* d_col_items[kBatchGroups] = {};
   int n_band[kBatchGroups] = {}, n_col[kBatchGroups] = {};
   std::vector<int2> h_band[kBatchGroups], h_col[kBatchGroups];
-  // the step-phase kernels (axpy, step) run over the bands of every 2-D slot; the sweeps
-  // (res, col, upd) over the slots without a one-launch inner solve, which run k_small_*_b on
-  // their own work lists (one entry per slot) in a parallel branch of the graph
+  // the band and column lists hold the 2-D slots that run the sweeps (res, col, upd) and their step
+  // phases (axpy, step); slots with a one-launch inner solve run k_small_*_b (one entry per slot)
+  // and their step phases over the bands of the phase list
   int2* d_phase_items[kBatchGroups] = {};
   int n_phase[kBatchGroups] = {};
   std::vector<int2> h_phase[kBatchGroups];
@@ -374,8 +374,11 @@ struct rd_batch {
   std::vector<int2> h_small[kBatchGroups][2];
   int smem_small[kBatchGroups][2] = {};
   int smem_usable = 0;
-  cudaStream_t fork_stream = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // one capture stream and join event per branch of the graph (see rebuild_graph)
+  cudaStream_t branch_stream[3 * kBatchGroups] = {};
+  cudaEvent_t ev_join[3 * kBatchGroups] = {};
+  cudaEvent_t ev_fork = nullptr;
+  int stale = 0;  // slots of the current work lists that have been retired
   // 3-D slots: one work list of (slot, block) pairs per group, and the largest transform-pass
   // block and shared memory any of its slots needs
   int2* d_items3[kBatchGroups] = {};
@@ -453,54 +456,54 @@ cudaError_t allow_batch_kernels(int optin) {
                               optin - (int)fa.sharedSizeBytes);
 }
 
+// The chain of one graph iteration for part `part` of group g (0: the slots that run the sweeps,
+// 1: the slots with a one-launch inner solve, 2: the 3-D slots).
 template <int K>
-void launch_group(rd_batch* b, int g, cudaStream_t s) {
-  const int np = b->n_phase[g], nb = b->n_band[g], ncl = b->n_col[g];
-  if (np == 0) return;
-  const int smem_res = KT<K>::two ? b->smem_sweep2 : b->smem_sweep, smem_col = b->smem_sweep;
-  k_axpy_b<<<np, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_phase_items[g]);
-  k_step_b<K><<<np, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_phase_items[g]);
-  const bool fork = b->n_small[g][0] + b->n_small[g][1] > 0;
-  if (fork) {
-    // the one-launch inner solves of the small slots, beside the sweeps of the others
-    cudaEventRecord(b->ev_fork, s);
-    cudaStreamWaitEvent(b->fork_stream, b->ev_fork, 0);
-    for (int m = 0; m < 2; ++m)
-      launch_small_batch(K, m + 1, b->d_d32, b->d_slots, b->d_small_items[g][m], b->n_small[g][m], b->smem_small[g][m],
-                         b->fork_stream);
-    cudaEventRecord(b->ev_join, b->fork_stream);
-  }
-  if (nb) {
+void launch_group(rd_batch* b, int g, int part, cudaStream_t s) {
+  if (part == 0) {
+    const int nb = b->n_band[g], ncl = b->n_col[g];
+    const int smem_res = KT<K>::two ? b->smem_sweep2 : b->smem_sweep, smem_col = b->smem_sweep;
+    k_axpy_b<<<nb, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_band_items[g]);
+    k_step_b<K><<<nb, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_band_items[g]);
     k_res_b<float, K><<<nb, kBatchThreads, smem_res, s>>>(b->d_d32, b->d_slots, b->d_band_items[g]);
     k_col_b<float><<<ncl, kBatchThreads, smem_col, s>>>(b->d_d32, b->d_slots, b->d_col_items[g]);
     k_upd_b<float, K><<<nb, kBatchThreads, smem_res, s>>>(b->d_d32, b->d_slots, b->d_band_items[g]);
+    return;
   }
-  if (fork) cudaStreamWaitEvent(s, b->ev_join, 0);
+  const int np = b->n_phase[g];
+  k_axpy_b<<<np, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_phase_items[g]);
+  k_step_b<K><<<np, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_phase_items[g]);
+  for (int m = 0; m < 2; ++m)
+    launch_small_batch(K, m + 1, b->d_d32, b->d_slots, b->d_small_items[g][m], b->n_small[g][m], b->smem_small[g][m], s);
 }
 
-void launch_iteration_all(rd_batch* b, cudaStream_t s) {
-  for (int g = 0; g < kBatchGroups; ++g) {
-    switch (kGroupKey[g]) {
-      case KK_NONE_LAP: launch_group<KK_NONE_LAP>(b, g, s); break;
-      case KK_AC: launch_group<KK_AC>(b, g, s); break;
-      case KK_CH_IMPL: launch_group<KK_CH_IMPL>(b, g, s); break;
-      case KK_CH_SPLIT: launch_group<KK_CH_SPLIT>(b, g, s); break;
-      case KK_GS: launch_group<KK_GS>(b, g, s); break;
-      case KK_SCHNAK: launch_group<KK_SCHNAK>(b, g, s); break;
-      default: launch_group<KK_NONE_BIH>(b, g, s); break;
+void launch_branch(rd_batch* b, int g, int part, cudaStream_t s) {
+  if (part == 2) {
+    Batch3Launch L{b->d_d32, b->d_d64, b->d_slots, b->d_items3[g], b->n_items3[g], {}, {}};
+    for (int a = 0; a < 3; ++a) {
+      L.thr[a] = b->thr3[g][a];
+      L.smem[a] = b->smem3[g][a];
     }
-    if (b->n_items3[g]) {
-      Batch3Launch L{b->d_d32, b->d_d64, b->d_slots, b->d_items3[g], b->n_items3[g], {}, {}};
-      for (int a = 0; a < 3; ++a) {
-        L.thr[a] = b->thr3[g][a];
-        L.smem[a] = b->smem3[g][a];
-      }
-      batch3_launch_group(kGroupKey[g], L, s);
-    }
+    batch3_launch_group(kGroupKey[g], L, s);
+    return;
+  }
+  switch (kGroupKey[g]) {
+    case KK_NONE_LAP: launch_group<KK_NONE_LAP>(b, g, part, s); break;
+    case KK_AC: launch_group<KK_AC>(b, g, part, s); break;
+    case KK_CH_IMPL: launch_group<KK_CH_IMPL>(b, g, part, s); break;
+    case KK_CH_SPLIT: launch_group<KK_CH_SPLIT>(b, g, part, s); break;
+    case KK_GS: launch_group<KK_GS>(b, g, part, s); break;
+    case KK_SCHNAK: launch_group<KK_SCHNAK>(b, g, part, s); break;
+    default: launch_group<KK_NONE_BIH>(b, g, part, s); break;
   }
 }
 
-// (Re)capture the graph of graph_k iterations over the current work lists.
+// (Re)capture the graph of graph_k iterations over the current work lists.  Slots of different
+// groups, and the sweep, one-launch and 3-D slots of one group, share nothing: each such part is a
+// branch of its own through all its iterations, so that the kernels of one fill the launch gaps and
+// idle SMs of the others (one chain through all of them: 28 launches in a row per iteration of a mix
+// of two kinds with cubes).  An iteration of the one-launch slots is a whole inner solve, as long as
+// several sweeps: their branch has a quarter of the iterations, so that no branch waits long for it.
 rd_status rebuild_graph(rd_batch* b) {
   if (b->gexec) {
     cudaGraphExecDestroy(b->gexec);
@@ -510,9 +513,28 @@ rd_status rebuild_graph(rd_batch* b) {
     cudaGraphDestroy(b->graph);
     b->graph = nullptr;
   }
-  cudaError_t e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
+  cudaError_t e = cudaSuccess;
+  std::vector<int> live;
+  for (int k = 0; k < 3 * kBatchGroups; ++k) {
+    const int g = k / 3, part = k % 3;
+    if ((part == 0 ? b->n_band[g] : part == 1 ? b->n_phase[g] : b->n_items3[g]) == 0) continue;
+    live.push_back(k);
+    if (!b->branch_stream[k]) e = cudaStreamCreateWithFlags(&b->branch_stream[k], cudaStreamNonBlocking);
+    if (e == cudaSuccess && !b->ev_join[k]) e = cudaEventCreateWithFlags(&b->ev_join[k], cudaEventDisableTiming);
+    if (e != cudaSuccess) return bfail(RD_ERR_CUDA, std::string("batch branches: ") + cudaGetErrorString(e));
+  }
+  e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return bfail(RD_ERR_CUDA, std::string("batch capture: ") + cudaGetErrorString(e));
-  for (int k = 0; k < b->opts.graph_k; ++k) launch_iteration_all(b, b->cap_stream);
+  cudaEventRecord(b->ev_fork, b->cap_stream);
+  for (int k : live) {
+    const int part = k % 3;
+    cudaStream_t s = b->branch_stream[k];
+    cudaStreamWaitEvent(s, b->ev_fork, 0);
+    const int iters = part == 1 ? std::max(1, b->opts.graph_k / 4) : b->opts.graph_k;
+    for (int i = 0; i < iters; ++i) launch_branch(b, k / 3, part, s);
+    cudaEventRecord(b->ev_join[k], s);
+    cudaStreamWaitEvent(b->cap_stream, b->ev_join[k], 0);
+  }
   cudaError_t el = cudaGetLastError();
   e = cudaStreamEndCapture(b->cap_stream, &b->graph);
   if (el != cudaSuccess || e != cudaSuccess)
@@ -550,9 +572,9 @@ rd_status rebuild_items(rd_batch* b) {
       }
       continue;
     }
-    for (int band = 0; band < sh.d32.nbands; ++band) b->h_phase[sh.group].push_back(make_int2(s, band));
     if (sh.small) {
       const Desc& d = sh.d32;
+      for (int band = 0; band < d.nbands; ++band) b->h_phase[sh.group].push_back(make_int2(s, band));
       const int m = sh.small - 1;
       b->h_small[sh.group][m].push_back(make_int2(s, 0));
       b->smem_small[sh.group][m] = std::max(
@@ -597,6 +619,7 @@ rd_status rebuild_items(rd_batch* b) {
     }
   }
   b->graph_dirty = true;
+  b->stale = 0;
   return RD_OK;
 }
 
@@ -1100,16 +1123,22 @@ void worker_loop(rd_batch* b) {
       std::lock_guard<std::mutex> lk(b->mu);
       b->stats.graph_launches += 1;
     }
-    bool retired = false;
+    int retired = 0, running = 0;
     for (int s = 0; s < b->max_slots; ++s) {
       if (!b->slots[s].used) continue;
       const Slot ctl = b->h_slots[s];
       if (ctl.phase == PH_DONE || ctl.phase == PH_FAILED) {
         retire(b, s, ctl);
-        retired = true;
+        ++retired;
+      } else {
+        ++running;
       }
     }
-    if (retired) rebuild_items(b);
+    // the blocks of a retired slot return at once (its control block is idle), so the lists and the
+    // graph, whose capture takes as long as several sweeps, stay until half their slots are gone (or
+    // a request is admitted)
+    b->stale += retired;
+    if (retired && running > 0 && b->stale >= running) rebuild_items(b);
   }
 }
 
@@ -1137,9 +1166,7 @@ rd_status rd_batch_create(rd_batch** out, size_t hbm_budget_bytes, int max_slots
   };
   cudaError_t e;
   if ((e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-      (e = cudaStreamCreateWithFlags(&b->fork_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-      (e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
-      (e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming)) != cudaSuccess)
+      (e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming)) != cudaSuccess)
     return cleanup(bfail(RD_ERR_CUDA, cudaGetErrorString(e)));
   if ((e = cudaMalloc(&b->arena_mem, hbm_budget_bytes)) != cudaSuccess) {
     cudaGetLastError();
@@ -1298,9 +1325,11 @@ void rd_batch_destroy(rd_batch* b) {
   if (b->h_slots) cudaFreeHost(b->h_slots);
   if (b->arena_mem) cudaFree(b->arena_mem);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-  if (b->fork_stream) cudaStreamDestroy(b->fork_stream);
+  for (cudaStream_t s : b->branch_stream)
+    if (s) cudaStreamDestroy(s);
+  for (cudaEvent_t ev : b->ev_join)
+    if (ev) cudaEventDestroy(ev);
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-  if (b->ev_join) cudaEventDestroy(b->ev_join);
   delete b;
 }
 
