@@ -167,11 +167,14 @@ struct BandThreads { static constexpr int value = sizeof(T) == 8 && V == 16 ? 25
 // of k_fcol: FP32 lines of 4096 and 8192 points take 1024 threads (at 64 registers, without spills
 // once the boundary kind is fixed at compile time) to hold two lines or more
 template <class T, int LOGN, int V>
-struct ColThreads { static constexpr int value = LOGN >= 12 && sizeof(T) == 4 ? 1024 : BandThreads<T, V>::value; };
+struct ColThreads {
+  static constexpr int value = LOGN >= 12 && sizeof(T) == 4 ? 1024 : BandThreads<T, V>::value;
+  static constexpr int blocks = sizeof(T) == 4 && V == 16 && LOGN == 11 ? 2 : 1;
+};
 
 // st = nullptr: the preconditioner alone, whatever the solve's state
 template <class T, int LOGN, int V, bool PER>
-__global__ void __launch_bounds__(ColThreads<T, LOGN, V>::value) k_fcol(const __grid_constant__ Desc d, State* __restrict__ st) {
+__global__ void __launch_bounds__(ColThreads<T, LOGN, V>::value, ColThreads<T, LOGN, V>::blocks) k_fcol(const __grid_constant__ Desc d, State* __restrict__ st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
   if (st && !sweep_active(st, nullptr)) return;
@@ -452,6 +455,15 @@ __host__ __device__ inline int primal_smem_bytes(int nc, int rows, int H, int nx
   return u > l ? u : l;
 }
 
+// Threads of a k_primal block at most, and the blocks an SM shall hold (the register cap): FP32 lines of
+// 4096 and 8192 points take 1024 threads; FP32 five-point kinds at V = 16 two blocks of 512 (64
+// registers, up to 100 bytes spilled for two species); the thirteen-point kinds would spill more.
+template <class T, int K, int LOGN, int V>
+struct PrimalBlock {
+  static constexpr int threads = sizeof(T) == 4 && LOGN >= 12 ? 1024 : BandThreads<T, V>::value;
+  static constexpr int blocks = sizeof(T) == 4 && V == 16 && LOGN < 12 && !KT<K>::biharm ? 2 : 1;
+};
+
 template <class T, int K, int LOGN, int V>
 __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ st, int band, bool first,
                                             unsigned char* smem_raw) {
@@ -620,7 +632,7 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
 }
 
 template <class T, int K, int LOGN, int V>
-__global__ void __launch_bounds__(BandThreads<T, V>::value) k_primal(const __grid_constant__ Desc d, State* __restrict__ st,
+__global__ void __launch_bounds__(PrimalBlock<T, K, LOGN, V>::threads, PrimalBlock<T, K, LOGN, V>::blocks) k_primal(const __grid_constant__ Desc d, State* __restrict__ st,
                                                                  int first) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();

@@ -765,9 +765,15 @@ bool plan_long(int nx, int ny, int nc, int H, bool neumann, Desc& d, LaunchCfg& 
   (void)neumann;
   Desc p = d;
   LaunchCfg q{};
-  p.band_rows = p.upd_rows = 2;
-  p.nbands = p.nupd = ny / 2;
   q.transform = 1;
+  p.col_width = 2;
+  for (int rows : {4, 2}) {
+    if (rows > ny) continue;
+    p.band_rows = p.upd_rows = rows;
+    p.nbands = p.nupd = ny / rows;
+    plan_band<T>(p, H, kSmemLimit, q);
+    if (q.fast_row) break;
+  }
   for (p.col_width = std::min(nx, 32 / (int)sizeof(T)); p.col_width >= 4; p.col_width /= 2) {
     plan_band<T>(p, H, kSmemLimit, q);
     if (q.fast_col && q.fast_row) break;
