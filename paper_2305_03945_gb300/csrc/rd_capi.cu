@@ -1152,16 +1152,15 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
   State sts[3] = {st, st, st};
   RD_CUDA(cudaMemcpy(h->d_state, sts, sizeof(sts), cudaMemcpyHostToDevice));
 
-  int usable = 0;
-  if (h->dc) RD_CUDA(set_kernel_smem_limits<float>(&usable));
-  else RD_CUDA(set_kernel_smem_limits<double>(&usable));
+  // shared memory: limits are raised for the kernels this handle launches (raising one loads its code)
+  int dev = 0, optin = 0;
+  RD_CUDA(cudaGetDevice(&dev));
+  RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const int usable = optin - 1024;
   if (h->nd3) {
-    int dev = 0, optin = 0;
-    RD_CUDA(cudaGetDevice(&dev));
-    RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    RD_CUDA(h->dc ? allow3<float>(optin) : allow3<double>(optin));
-    if (h->cube.on) RD_CUDA(allow_cube(d32, h->cube, optin));
-    RD_CUDA(allow3<double>(optin));  // the preconditioner-only solve of rd_pdhg_apply_precond
+    if (!h->dc) RD_CUDA(allow3<double>(optin));
+    else if (h->cube.on) RD_CUDA(allow_cube(d32, h->cube, optin));
+    else RD_CUDA(allow3<float>(optin));
   }
   const LaunchCfg& lc = h->dc ? h->cfg32 : h->cfg64;
   if (std::max(lc.smem_res, std::max(lc.smem_col, lc.smem_upd)) > usable)
@@ -1173,12 +1172,7 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
                               rx->kind == RD_RX_NONE ? (op == RD_OP_NEG_BIHARMONIC ? KK_NONE_BIH : KK_NONE_LAP) : rx->kind,
                               bc == RD_BC_NEUMANN, usable)
                  : 0;
-  if (h->small) {
-    int dev = 0, optin = 0;
-    RD_CUDA(cudaGetDevice(&dev));
-    RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    RD_CUDA(allow_small(optin));
-  }
+  if (h->small) RD_CUDA(allow_small_solve(h->h_desc[1], h->small, optin));
   if (!h->nd3 && !h->small) {
     const int ti = h->dc ? 1 : 0;
     Desc& d = h->h_desc[ti];
@@ -1191,9 +1185,6 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
       }
     }
     const bool fused = may_fuse && c.fast_row;
-    int dev = 0, optin = 0;
-    RD_CUDA(cudaGetDevice(&dev));
-    RD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     if (!h->dc && c.fast_col) {
       RD_TRY(dalloc(h, &h->sym64, h->npts * sizeof(double)));
       RD_CUDA(launch_symbol(d, h->sym64, h->stream));
@@ -1201,7 +1192,10 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
     }
     RD_CUDA(h->dc ? allow_band<float>(d, c, optin, fused) : allow_band<double>(d, c, optin, fused));
     if (!h->dc) h->cfgpc = c;
-    if (h->fch && fch_fused(h->cfgpc)) RD_CUDA(allow_fch(d, h->cfgpc, optin));
+    const bool fch_new = h->fch && fch_fused(h->cfgpc);
+    if (fch_new) RD_CUDA(allow_fch(d, h->cfgpc, optin));
+    if (!fch_new && !(fused && c.fast_col))
+      RD_CUDA(h->dc ? set_kernel_smem_limits<float>(nullptr) : set_kernel_smem_limits<double>(nullptr));
     share_tiles(h, d);
     if (h->opts.autotune && !h->fch && !h->long2d && h->opts.band_rows == 0 && h->opts.col_width == 0 && h->opts.upd_rows == 0) {
       const int stage_base = h->dc && (rx->kind == RD_RX_CH_IMPLICIT || rx->kind == RD_RX_CH_SPLIT);

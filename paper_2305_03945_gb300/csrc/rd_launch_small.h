@@ -19,7 +19,9 @@ cudaError_t launch_small(const Desc& d, State* st, int mode, cudaStream_t s);
 // (slot, 0); smem = the largest slot's bytes.
 cudaError_t launch_small_batch(int key, int mode, const Desc* descs, Slot* slots, const int2* items, int nitems,
                                int smem, cudaStream_t s);
-// Raise the dynamic shared-memory limit of the small-solve kernels.
+// Raise the dynamic shared-memory limit of the kernel that launch_small launches for d, and of the
+// batched ones.
+cudaError_t allow_small_solve(const Desc& d, int mode, int optin);
 cudaError_t allow_small(int optin);
 
 }  // namespace rd

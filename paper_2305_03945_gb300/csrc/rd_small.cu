@@ -131,27 +131,33 @@ cudaError_t launch_small_batch(int key, int mode, const Desc* descs, Slot* slots
   return cudaGetLastError();
 }
 
+namespace {
+template <int K>
+cudaError_t allow_one(int mode, int optin) {
+  return mode == 2 ? allow_k(k_small_cl<K>, optin) : allow_k(k_small<K>, optin);
+}
+}  // namespace
+
+cudaError_t allow_small_solve(const Desc& d, int mode, int optin) {
+  switch (kind_key(d)) {
+    case KK_NONE_LAP: return allow_one<KK_NONE_LAP>(mode, optin);
+    case KK_AC: return allow_one<KK_AC>(mode, optin);
+    case KK_CH_IMPL: return allow_one<KK_CH_IMPL>(mode, optin);
+    case KK_CH_SPLIT: return allow_one<KK_CH_SPLIT>(mode, optin);
+    case KK_GS: return allow_one<KK_GS>(mode, optin);
+    case KK_SCHNAK: return allow_one<KK_SCHNAK>(mode, optin);
+    case KK_NONE_BIH: return allow_one<KK_NONE_BIH>(mode, optin);
+    default: return cudaErrorNotSupported;
+  }
+}
+
 cudaError_t allow_small(int optin) {
   cudaError_t e;
-  if ((e = allow_k(k_small<KK_NONE_LAP>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small<KK_AC>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small<KK_CH_IMPL>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small<KK_CH_SPLIT>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small<KK_GS>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small<KK_SCHNAK>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small<KK_NONE_BIH>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_b<KK_NONE_LAP>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_b<KK_AC>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_b<KK_CH_IMPL>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_b<KK_CH_SPLIT>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_b<KK_NONE_BIH>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small_cl<KK_NONE_LAP>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small_cl<KK_AC>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small_cl<KK_CH_IMPL>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small_cl<KK_CH_SPLIT>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small_cl<KK_GS>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small_cl<KK_SCHNAK>, optin)) != cudaSuccess) return e;
-  if ((e = allow_k(k_small_cl<KK_NONE_BIH>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_cl_b<KK_NONE_LAP>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_cl_b<KK_AC>, optin)) != cudaSuccess) return e;
   if ((e = allow_k(k_small_cl_b<KK_CH_IMPL>, optin)) != cudaSuccess) return e;
