@@ -343,16 +343,15 @@ __global__ void __launch_bounds__(BandThreads<T, V>::value) k_rowfwd(const __gri
 // ---------------------------------------------------------------------------------------
 // k_dual
 // ---------------------------------------------------------------------------------------
+// The lines of group `grp` (blockDim.x / TPL row pairs of the stacked components and planes).  P~ may
+// overwrite Y (d.P[1] = d.WY): a line's coefficients are all read before its first store.
 template <class T, int LOGN, int V, bool PC>
-__global__ void __launch_bounds__(BandThreads<T, V>::value) k_dual(const __grid_constant__ Desc d, State* __restrict__ st) {
+__device__ __forceinline__ void dual_body(const Desc& d, int grp, unsigned char* smem_raw) {
   using F = Rf<LOGN, V>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_wait();
-  if (!PC && !sweep_active(st, nullptr)) return;
   constexpr int N = F::N;
   const int lline = threadIdx.x / F::TPL, t = threadIdx.x % F::TPL;
   const int lines = d.ncomp * (d.ny >> 1) * (d.nz > 1 ? d.nz : 1);
-  const int gl = blockIdx.x * (blockDim.x / F::TPL) + lline;
+  const int gl = grp * (blockDim.x / F::TPL) + lline;
   const bool live = gl < lines;
   cx<T>* line = reinterpret_cast<cx<T>*>(smem_raw) + lline * Lay<T, LOGN, V, false>::len;
   const bool per = d.bc == BC_PERIODIC;
@@ -400,6 +399,14 @@ __global__ void __launch_bounds__(BandThreads<T, V>::value) k_dual(const __grid_
       st4(Pt + N + j0, pb[i]);
     }
   }
+}
+
+template <class T, int LOGN, int V, bool PC>
+__global__ void __launch_bounds__(BandThreads<T, V>::value) k_dual(const __grid_constant__ Desc d, State* __restrict__ st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_wait();
+  if (!PC && !sweep_active(st, nullptr)) return;
+  dual_body<T, LOGN, V, PC>(d, blockIdx.x, smem_raw);
 }
 
 // ---------------------------------------------------------------------------------------

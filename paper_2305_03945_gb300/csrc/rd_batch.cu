@@ -31,6 +31,7 @@
 #include "../../include/rd_pdhg.h"
 #include "rd_3d.cuh"
 #include "rd_batch3.h"
+#include "rd_batch_lines.h"
 #include "rd_launch3.h"
 #include "rd_launch_small.h"
 
@@ -249,6 +250,7 @@ constexpr int kBatchMaxBlk3 = 1024;     // blocks per 3-D slot (plan3's cap)
 constexpr int kBatchBandRows = 4;
 constexpr int kBatchColWidth = 4;
 constexpr int kBatchGroups = 7;         // equation kinds served
+constexpr int kBatchParts = 5;          // branches of a group's graph: see launch_branch
 const int kGroupKey[kBatchGroups] = {KK_NONE_LAP, KK_AC, KK_CH_IMPL, KK_CH_SPLIT, KK_NONE_BIH, KK_GS, KK_SCHNAK};
 
 double now_s() {
@@ -301,6 +303,28 @@ struct Arena {
   }
 };
 
+// A work list of (slot, block) pairs: built on the host, copied to a device array that grows to fit.
+struct ItemList {
+  int2* d = nullptr;
+  int cap = 0, n = 0;
+  std::vector<int2> h;
+  cudaError_t upload(cudaStream_t s) {
+    n = (int)h.size();
+    if (n == 0) return cudaSuccess;
+    if (n > cap) {
+      if (d) cudaFree(d);
+      d = nullptr;
+      cap = std::max(2 * n, 1024);
+      const cudaError_t e = cudaMalloc(&d, sizeof(int2) * cap);
+      if (e != cudaSuccess) {
+        cap = 0;
+        return e;
+      }
+    }
+    return cudaMemcpyAsync(d, h.data(), n * sizeof(int2), cudaMemcpyHostToDevice, s);
+  }
+};
+
 struct Request {
   uint64_t id = 0;
   rd_request req{};
@@ -317,7 +341,8 @@ struct SlotHost {
   size_t mem_bytes = 0;
   size_t npts = 0;
   double t_submit = 0, t_admit = 0;
-  bool nd3 = false;  // a 3-D request (the rd_batch3.cu kernels)
+  bool nd3 = false;  // a 3-D request
+  bool fast = false; // every side 16 points or more: the line kernels of rd_batch_lines.cuh
   int small = 0;     // a 2-D request whose inner solves run in one launch (1 one block, 2 a cluster)
   Desc d32{}, d64{};
 };
@@ -359,40 +384,34 @@ struct rd_batch {
   Desc* d_d64 = nullptr;
   Slot* d_slots = nullptr;
   Slot* h_slots = nullptr;  // pinned mirror
-  int2* d_band_items[kBatchGroups] = {};
-  int2* d_col_items[kBatchGroups] = {};
-  int n_band[kBatchGroups] = {}, n_col[kBatchGroups] = {};
-  std::vector<int2> h_band[kBatchGroups], h_col[kBatchGroups];
-  // the band and column lists hold the 2-D slots that run the sweeps (res, col, upd) and their step
-  // phases (axpy, step); slots with a one-launch inner solve run k_small_*_b (one entry per slot)
-  // and their step phases over the bands of the phase list
-  int2* d_phase_items[kBatchGroups] = {};
-  int n_phase[kBatchGroups] = {};
-  std::vector<int2> h_phase[kBatchGroups];
-  int2* d_small_items[kBatchGroups][2] = {};
-  int n_small[kBatchGroups][2] = {};
-  std::vector<int2> h_small[kBatchGroups][2];
-  int smem_small[kBatchGroups][2] = {};
+  // Work lists per group.  Slots with a one-launch inner solve: one entry per slot in small1 / small2
+  // (one block / a cluster each) and the bands of their step phases (axpy, step) in small_phase.  2-D
+  // slots: bands and column blocks of the Stockham sweeps (band, col), or, with line kernels, the bands
+  // of the step phases and the blocks of the line kernels (line_phase, line2).  3-D slots: blocks of
+  // either set of kernels (old3, line3).
+  struct Lists {
+    ItemList band, col, small_phase, small1, small2, line_phase, line2, old3, line3;
+    int smem_small[2] = {};
+    int smem_line2[2] = {}, smem_line3[2] = {};  // row and column kernels
+    int thr3[3] = {}, smem3[3] = {};             // transform passes of the old3 slots
+  } lists[kBatchGroups];
   int smem_usable = 0;
   // one capture stream and join event per branch of the graph (see rebuild_graph)
-  cudaStream_t branch_stream[3 * kBatchGroups] = {};
-  cudaEvent_t ev_join[3 * kBatchGroups] = {};
+  cudaStream_t branch_stream[kBatchParts * kBatchGroups] = {};
+  cudaEvent_t ev_join[kBatchParts * kBatchGroups] = {};
   cudaEvent_t ev_fork = nullptr;
   int stale = 0;  // slots of the current work lists that have been retired
-  // 3-D slots: one work list of (slot, block) pairs per group, and the largest transform-pass
-  // block and shared memory any of its slots needs
-  int2* d_items3[kBatchGroups] = {};
-  int n_items3[kBatchGroups] = {};
-  std::vector<int2> h_items3[kBatchGroups];
-  int thr3[kBatchGroups][3] = {}, smem3[kBatchGroups][3] = {};
+  // twiddle and DCT rotation tables of every line length 4 .. kBatchMaxSide, shared by all slots: those
+  // of length n at n - 4 complex entries each (twiddles), and behind all of them (rotations); sines of
+  // pi k / (2 kBatchMaxSide) for the eigenvalues
+  cx<float>* d_tables = nullptr;
+  std::vector<double> sines;
   std::vector<SlotHost> slots;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   bool graph_dirty = true;
   int smem_sweep = 0;
   int smem_sweep2 = 0;  // the band kernels of the two-species kinds
-  // measured tiles per grid size (index log2 of the longer side; 0 = not measured)
-  int tune_band[16] = {}, tune_col[16] = {};
   // queues.  mu guards the queues, outputs, stats, worker_error, stop and the arena's free list
   // (allocated and released by the worker, read by rd_batch_get_stats); never held across a
   // CUDA call that waits on the device.
@@ -426,20 +445,40 @@ int group_of(int key) {
   return -1;
 }
 
-void host_tables(int n, bool neumann, double h, std::vector<float>& tw, std::vector<float>& dc, std::vector<float>& mu) {
+// Tables of every line length, once per batch: one pass of long double trigonometry (software on this
+// host) for all admissions.  w_n^k = w_N^{k N/n} with N = kBatchMaxSide, an exact scaling of the argument.
+rd_status make_tables(rd_batch* b) {
   const long double pi = 3.141592653589793238462643383279502884L;
-  tw.resize(2 * n);
-  dc.resize(2 * n);
-  mu.resize(n);
+  constexpr int N = kBatchMaxSide;
+  b->sines.resize(2 * N + 1);
+  std::vector<cx<float>> tab(2 * (2 * N - 4));
+  std::vector<cx<float>> tw(N), dc(N);
+  for (int k = 0; k < N; ++k) {
+    const long double t = 2.0L * pi * k / N;
+    tw[k] = cx<float>{(float)cosl(t), (float)(-sinl(t))};
+    const long double q = pi * k / (2.0L * N);
+    dc[k] = cx<float>{(float)cosl(q), (float)sinl(q)};
+  }
+  for (int k = 0; k <= 2 * N; ++k) b->sines[k] = (double)sinl(pi * k / (2.0L * N));
+  for (int n = 4; n <= N; n *= 2)
+    for (int k = 0; k < n; ++k) {
+      tab[n - 4 + k] = tw[k * (N / n)];
+      tab[2 * N - 4 + n - 4 + k] = dc[k * (N / n)];
+    }
+  cudaError_t e = cudaMalloc(&b->d_tables, tab.size() * sizeof(cx<float>));
+  if (e == cudaSuccess) e = cudaMemcpy(b->d_tables, tab.data(), tab.size() * sizeof(cx<float>), cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? RD_OK : bfail(RD_ERR_OOM, std::string("batch tables: ") + cudaGetErrorString(e));
+}
+
+const cx<float>* twiddles_of(const rd_batch* b, int n) { return b->d_tables + (n - 4); }
+const cx<float>* rotations_of(const rd_batch* b, int n) { return b->d_tables + (2 * kBatchMaxSide - 4) + (n - 4); }
+
+// eigenvalues of -Lap along one axis, mu(k) = 4/h^2 sin^2(pi k / (d n)), d = 1 periodic, 2 Neumann
+void append_mu(const rd_batch* b, int n, bool neumann, double h, std::vector<float>& mu) {
+  const int step = (neumann ? 1 : 2) * (kBatchMaxSide / n);
   for (int k = 0; k < n; ++k) {
-    const long double t = 2.0L * pi * k / n;
-    tw[2 * k] = (float)cosl(t);
-    tw[2 * k + 1] = (float)(-sinl(t));
-    const long double q = pi * k / (2.0L * n);
-    dc[2 * k] = (float)cosl(q);
-    dc[2 * k + 1] = (float)sinl(q);
-    const long double sn = sinl(pi * k / ((neumann ? 2.0L : 1.0L) * n));
-    mu[k] = (float)(4.0L / ((long double)h * h) * sn * sn);
+    const double sn = b->sines[k * step];
+    mu.push_back((float)(4.0 / (h * h) * sn * sn));
   }
 }
 
@@ -456,35 +495,50 @@ cudaError_t allow_batch_kernels(int optin) {
                               optin - (int)fa.sharedSizeBytes);
 }
 
-// The chain of one graph iteration for part `part` of group g (0: the slots that run the sweeps,
-// 1: the slots with a one-launch inner solve, 2: the 3-D slots).
+// The chain of one graph iteration for part `part` of group g: 0 the 2-D slots on the Stockham sweeps,
+// 1 the slots with a one-launch inner solve, 2 the 3-D slots on the Stockham passes, 3 and 4 the 2-D and
+// 3-D slots on the line kernels.
 template <int K>
 void launch_group(rd_batch* b, int g, int part, cudaStream_t s) {
+  const rd_batch::Lists& l = b->lists[g];
+  const ItemList& ph = part == 0 ? l.band : (part == 1 ? l.small_phase : l.line_phase);
+  k_axpy_b<<<ph.n, 256, 0, s>>>(b->d_d64, b->d_slots, ph.d);
+  k_step_b<K><<<ph.n, 256, 0, s>>>(b->d_d64, b->d_slots, ph.d);
   if (part == 0) {
-    const int nb = b->n_band[g], ncl = b->n_col[g];
     const int smem_res = KT<K>::two ? b->smem_sweep2 : b->smem_sweep, smem_col = b->smem_sweep;
-    k_axpy_b<<<nb, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_band_items[g]);
-    k_step_b<K><<<nb, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_band_items[g]);
-    k_res_b<float, K><<<nb, kBatchThreads, smem_res, s>>>(b->d_d32, b->d_slots, b->d_band_items[g]);
-    k_col_b<float><<<ncl, kBatchThreads, smem_col, s>>>(b->d_d32, b->d_slots, b->d_col_items[g]);
-    k_upd_b<float, K><<<nb, kBatchThreads, smem_res, s>>>(b->d_d32, b->d_slots, b->d_band_items[g]);
-    return;
+    k_res_b<float, K><<<l.band.n, kBatchThreads, smem_res, s>>>(b->d_d32, b->d_slots, l.band.d);
+    k_col_b<float><<<l.col.n, kBatchThreads, smem_col, s>>>(b->d_d32, b->d_slots, l.col.d);
+    k_upd_b<float, K><<<l.band.n, kBatchThreads, smem_res, s>>>(b->d_d32, b->d_slots, l.band.d);
+  } else if (part == 1) {
+    launch_small_batch(K, 1, b->d_d32, b->d_slots, l.small1.d, l.small1.n, l.smem_small[0], s);
+    launch_small_batch(K, 2, b->d_d32, b->d_slots, l.small2.d, l.small2.n, l.smem_small[1], s);
+  } else {
+    batch_lines2(K, BatchLines{b->d_d32, b->d_slots, l.line2.d, l.line2.n, l.smem_line2[0], l.smem_line2[1]}, s);
   }
-  const int np = b->n_phase[g];
-  k_axpy_b<<<np, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_phase_items[g]);
-  k_step_b<K><<<np, 256, 0, s>>>(b->d_d64, b->d_slots, b->d_phase_items[g]);
-  for (int m = 0; m < 2; ++m)
-    launch_small_batch(K, m + 1, b->d_d32, b->d_slots, b->d_small_items[g][m], b->n_small[g][m], b->smem_small[g][m], s);
+}
+
+// entries of the list that decides whether a part has work
+int part_items(const rd_batch* b, int g, int part) {
+  const rd_batch::Lists& l = b->lists[g];
+  const ItemList* of[kBatchParts] = {&l.band, &l.small_phase, &l.old3, &l.line2, &l.line3};
+  return of[part]->n;
 }
 
 void launch_branch(rd_batch* b, int g, int part, cudaStream_t s) {
-  if (part == 2) {
-    Batch3Launch L{b->d_d32, b->d_d64, b->d_slots, b->d_items3[g], b->n_items3[g], {}, {}};
+  const rd_batch::Lists& l = b->lists[g];
+  if (part == 2 || part == 4) {
+    const ItemList& it = part == 2 ? l.old3 : l.line3;
+    Batch3Launch L{b->d_d32, b->d_d64, b->d_slots, it.d, it.n, {}, {}};
     for (int a = 0; a < 3; ++a) {
-      L.thr[a] = b->thr3[g][a];
-      L.smem[a] = b->smem3[g][a];
+      L.thr[a] = l.thr3[a];
+      L.smem[a] = l.smem3[a];
     }
-    batch3_launch_group(kGroupKey[g], L, s);
+    if (part == 2) {
+      batch3_launch_group(kGroupKey[g], L, s);
+    } else {
+      batch3_launch_phases(kGroupKey[g], L, s);
+      batch_lines3(kGroupKey[g], BatchLines{b->d_d32, b->d_slots, it.d, it.n, l.smem_line3[0], l.smem_line3[1]}, s);
+    }
     return;
   }
   switch (kGroupKey[g]) {
@@ -515,9 +569,8 @@ rd_status rebuild_graph(rd_batch* b) {
   }
   cudaError_t e = cudaSuccess;
   std::vector<int> live;
-  for (int k = 0; k < 3 * kBatchGroups; ++k) {
-    const int g = k / 3, part = k % 3;
-    if ((part == 0 ? b->n_band[g] : part == 1 ? b->n_phase[g] : b->n_items3[g]) == 0) continue;
+  for (int k = 0; k < kBatchParts * kBatchGroups; ++k) {
+    if (part_items(b, k / kBatchParts, k % kBatchParts) == 0) continue;
     live.push_back(k);
     if (!b->branch_stream[k]) e = cudaStreamCreateWithFlags(&b->branch_stream[k], cudaStreamNonBlocking);
     if (e == cudaSuccess && !b->ev_join[k]) e = cudaEventCreateWithFlags(&b->ev_join[k], cudaEventDisableTiming);
@@ -527,11 +580,11 @@ rd_status rebuild_graph(rd_batch* b) {
   if (e != cudaSuccess) return bfail(RD_ERR_CUDA, std::string("batch capture: ") + cudaGetErrorString(e));
   cudaEventRecord(b->ev_fork, b->cap_stream);
   for (int k : live) {
-    const int part = k % 3;
+    const int part = k % kBatchParts;
     cudaStream_t s = b->branch_stream[k];
     cudaStreamWaitEvent(s, b->ev_fork, 0);
     const int iters = part == 1 ? std::max(1, b->opts.graph_k / 4) : b->opts.graph_k;
-    for (int i = 0; i < iters; ++i) launch_branch(b, k / 3, part, s);
+    for (int i = 0; i < iters; ++i) launch_branch(b, k / kBatchParts, part, s);
     cudaEventRecord(b->ev_join[k], s);
     cudaStreamWaitEvent(b->cap_stream, b->ev_join[k], 0);
   }
@@ -548,73 +601,50 @@ rd_status rebuild_graph(rd_batch* b) {
 // Upload the work lists of all groups from the slot table.
 rd_status rebuild_items(rd_batch* b) {
   for (int g = 0; g < kBatchGroups; ++g) {
-    b->h_band[g].clear();
-    b->h_col[g].clear();
-    b->h_phase[g].clear();
-    for (int m = 0; m < 2; ++m) {
-      b->h_small[g][m].clear();
-      b->smem_small[g][m] = 0;
-    }
-    b->h_items3[g].clear();
-    for (int a = 0; a < 3; ++a) b->thr3[g][a] = b->smem3[g][a] = 0;
+    rd_batch::Lists& l = b->lists[g];
+    for (ItemList* it : {&l.band, &l.col, &l.small_phase, &l.small1, &l.small2, &l.line_phase, &l.line2, &l.old3, &l.line3})
+      it->h.clear();
+    for (int m = 0; m < 2; ++m) l.smem_small[m] = l.smem_line2[m] = l.smem_line3[m] = 0;
+    for (int a = 0; a < 3; ++a) l.thr3[a] = l.smem3[a] = 0;
   }
   for (int s = 0; s < b->max_slots; ++s) {
     const SlotHost& sh = b->slots[s];
     if (!sh.used) continue;
-    if (sh.nd3) {
-      const Desc& d = sh.d32;
-      for (int k = 0; k < d.blk3; ++k) b->h_items3[sh.group].push_back(make_int2(s, k));
+    const Desc& d = sh.d32;
+    rd_batch::Lists& l = b->lists[sh.group];
+    auto list = [s](ItemList& it, int n) {
+      for (int k = 0; k < n; ++k) it.h.push_back(make_int2(s, k));
+    };
+    if (sh.fast) {
+      list(sh.nd3 ? l.line3 : l.line2, d.blk3);
+      if (!sh.nd3) list(l.line_phase, d.nbands);
+      int* sm = sh.nd3 ? l.smem_line3 : l.smem_line2;
+      int row = 0, col = 0;
+      if (sh.nd3) batch_lines3_plan(d, 1, &row, &col);
+      else batch_lines2_plan(d, 1, &row, &col);
+      sm[0] = std::max(sm[0], row);
+      sm[1] = std::max(sm[1], col);
+    } else if (sh.nd3) {
+      list(l.old3, d.blk3);
       const int n_ax[3] = {d.nx, d.ny, d.nz};
       for (int a = 0; a < 3; ++a) {
-        b->thr3[sh.group][a] = std::max(b->thr3[sh.group][a], d.thr3[a]);
-        b->smem3[sh.group][a] = std::max(b->smem3[sh.group][a],
-                                         lines3_smem_bytes<float>(n_ax[a], d.lw3[a], d.bc == BC_NEUMANN));
+        l.thr3[a] = std::max(l.thr3[a], d.thr3[a]);
+        l.smem3[a] = std::max(l.smem3[a], lines3_smem_bytes<float>(n_ax[a], d.lw3[a], d.bc == BC_NEUMANN));
       }
-      continue;
+    } else if (sh.small) {
+      list(l.small_phase, d.nbands);
+      list(sh.small == 1 ? l.small1 : l.small2, 1);
+      int& sm = l.smem_small[sh.small - 1];
+      sm = std::max(sm, small_smem_of(sh.small, d.nx, d.ny, d.ncomp, sh.key, d.bc == BC_NEUMANN));
+    } else {
+      list(l.band, d.nbands);
+      list(l.col, d.ncomp * d.ncolblk);
     }
-    if (sh.small) {
-      const Desc& d = sh.d32;
-      for (int band = 0; band < d.nbands; ++band) b->h_phase[sh.group].push_back(make_int2(s, band));
-      const int m = sh.small - 1;
-      b->h_small[sh.group][m].push_back(make_int2(s, 0));
-      b->smem_small[sh.group][m] = std::max(
-          b->smem_small[sh.group][m], small_smem_of(sh.small, d.nx, d.ny, d.ncomp, sh.key, d.bc == BC_NEUMANN));
-      continue;
-    }
-    for (int band = 0; band < sh.d32.nbands; ++band) b->h_band[sh.group].push_back(make_int2(s, band));
-    for (int cb = 0; cb < sh.d32.ncomp * sh.d32.ncolblk; ++cb) b->h_col[sh.group].push_back(make_int2(s, cb));
   }
   for (int g = 0; g < kBatchGroups; ++g) {
-    b->n_band[g] = (int)b->h_band[g].size();
-    b->n_col[g] = (int)b->h_col[g].size();
-    b->n_items3[g] = (int)b->h_items3[g].size();
-    b->n_phase[g] = (int)b->h_phase[g].size();
-    if (b->n_phase[g]) {
-      cudaError_t e = cudaMemcpyAsync(b->d_phase_items[g], b->h_phase[g].data(), b->n_phase[g] * sizeof(int2),
-                                      cudaMemcpyHostToDevice, b->stream);
-      if (e != cudaSuccess) return bfail(RD_ERR_CUDA, cudaGetErrorString(e));
-    }
-    for (int m = 0; m < 2; ++m) {
-      b->n_small[g][m] = (int)b->h_small[g][m].size();
-      if (b->n_small[g][m]) {
-        cudaError_t e = cudaMemcpyAsync(b->d_small_items[g][m], b->h_small[g][m].data(),
-                                        b->n_small[g][m] * sizeof(int2), cudaMemcpyHostToDevice, b->stream);
-        if (e != cudaSuccess) return bfail(RD_ERR_CUDA, cudaGetErrorString(e));
-      }
-    }
-    if (b->n_items3[g]) {
-      cudaError_t e = cudaMemcpyAsync(b->d_items3[g], b->h_items3[g].data(), b->n_items3[g] * sizeof(int2),
-                                      cudaMemcpyHostToDevice, b->stream);
-      if (e != cudaSuccess) return bfail(RD_ERR_CUDA, cudaGetErrorString(e));
-    }
-    if (b->n_band[g]) {
-      cudaError_t e = cudaMemcpyAsync(b->d_band_items[g], b->h_band[g].data(), b->n_band[g] * sizeof(int2),
-                                      cudaMemcpyHostToDevice, b->stream);
-      if (e != cudaSuccess) return bfail(RD_ERR_CUDA, cudaGetErrorString(e));
-    }
-    if (b->n_col[g]) {
-      cudaError_t e = cudaMemcpyAsync(b->d_col_items[g], b->h_col[g].data(), b->n_col[g] * sizeof(int2),
-                                      cudaMemcpyHostToDevice, b->stream);
+    rd_batch::Lists& l = b->lists[g];
+    for (ItemList* it : {&l.band, &l.col, &l.small_phase, &l.small1, &l.small2, &l.line_phase, &l.line2, &l.old3, &l.line3}) {
+      const cudaError_t e = it->upload(b->stream);
       if (e != cudaSuccess) return bfail(RD_ERR_CUDA, cudaGetErrorString(e));
     }
   }
@@ -642,7 +672,7 @@ void admit3(rd_batch* b, Request& q, int s, char* mem, size_t npts, rd_status* e
   float* wy = (float*)take(npts * 4);
   float* r32 = (float*)take(npts * 4);
   float* u32 = (float*)take(npts * 4);
-  float* tabs = (float*)take((size_t)(nx + ny + nz) * 2 * 8);
+  take((size_t)(nx + ny + nz) * 2 * 8);  // (the tables are the batch's; the request's size stays as it was)
   float* mus = (float*)take((size_t)(nx + ny + nz) * 4);
   double* parts = (double*)take((size_t)2 * kBatchMaxBlk3 * 8);
   const double hx = r.grid.length[0] / nx, hy = r.grid.length[1] / ny, hz = r.grid.length[2] / nz;
@@ -699,33 +729,28 @@ void admit3(rd_batch* b, Request& q, int s, char* mem, size_t npts, rd_status* e
   d32.P[0] = p0;
   d32.P[1] = p0;
   d32.WY = wy;
-  cx<float>* twx = reinterpret_cast<cx<float>*>(tabs);
-  cx<float>* dcx = twx + nx;
-  cx<float>* twy = dcx + nx;
-  cx<float>* dcy = twy + ny;
-  cx<float>* twz = dcy + ny;
-  cx<float>* dcz = twz + nz;
-  d32.twx = twx;
-  d32.dcx = dcx;
-  d32.twy = twy;
-  d32.dcy = dcy;
-  d32.twz = twz;
-  d32.dcz = dcz;
+  d32.twx = twiddles_of(b, nx);
+  d32.dcx = rotations_of(b, nx);
+  d32.twy = twiddles_of(b, ny);
+  d32.dcy = rotations_of(b, ny);
+  d32.twz = twiddles_of(b, nz);
+  d32.dcz = rotations_of(b, nz);
   d32.mux = mus;
   d32.muy = mus + nx;
   d32.muz = mus + nx + ny;
+  sh.fast = nx >= 16 && ny >= 16 && nz >= 16;
+  if (sh.fast) {
+    int row = 0, col = 0;
+    d32.blk3 = d64.blk3 = batch_lines3_plan(d32, kBatchMaxBlk3, &row, &col);
+    d32.P[1] = wy;
+  }
   sh.d32 = d32;
   sh.d64 = d64;
   sh.nd3 = true;
-  std::vector<float> tw, dc, mu, all_t, all_mu;
+  std::vector<float> all_mu;
   const int n_ax[3] = {nx, ny, nz};
   const double h_ax[3] = {hx, hy, hz};
-  for (int a = 0; a < 3; ++a) {
-    host_tables(n_ax[a], r.bc == RD_BC_NEUMANN, h_ax[a], tw, dc, mu);
-    all_t.insert(all_t.end(), tw.begin(), tw.end());
-    all_t.insert(all_t.end(), dc.begin(), dc.end());
-    all_mu.insert(all_mu.end(), mu.begin(), mu.end());
-  }
+  for (int a = 0; a < 3; ++a) append_mu(b, n_ax[a], r.bc == RD_BC_NEUMANN, h_ax[a], all_mu);
   Slot ctl{};
   ctl.outer.max_iter = 1 << 30;
   ctl.inner.max_iter = b->opts.max_iter;
@@ -737,14 +762,12 @@ void admit3(rd_batch* b, Request& q, int s, char* mem, size_t npts, rd_status* e
   ctl.tol_kind = r.tol_kind;
   cudaStream_t st = b->stream;
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(tabs, all_t.data(), all_t.size() * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(mus, all_mu.data(), all_mu.size() * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(u, q.u0.data(), npts * 8, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d32 + s, &sh.d32, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d64 + s, &sh.d64, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_slots + s, &ctl, sizeof(Slot), cudaMemcpyHostToDevice, st);
-  // the host vectors above are pageable: wait for the copies before they go out of scope
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  // (no wait: the copies read pageable memory, which cudaMemcpyAsync has staged when it returns)
   if (e != cudaSuccess) *err = bfail(RD_ERR_CUDA, std::string("admission: ") + cudaGetErrorString(e));
 }
 
@@ -777,7 +800,7 @@ bool admit(rd_batch* b, Request& q, rd_status* err) {
   sh.npts = npts;
   sh.t_submit = q.t_submit;
   sh.t_admit = now_s();
-  sh.nd3 = false;
+  sh.nd3 = sh.fast = false;
   if (q.req.grid.ndim == 3) {
     admit3(b, q, s, mem, npts, err);
     std::lock_guard<std::mutex> lk(b->mu);
@@ -800,7 +823,7 @@ bool admit(rd_batch* b, Request& q, rd_status* err) {
   float* wy = (float*)take(npts * 4);
   float* r32 = (float*)take(npts * 4);
   float* u32 = (float*)take(npts * 4);
-  float* tabs = (float*)take((size_t)(nx + ny) * 2 * 8);
+  take((size_t)(nx + ny) * 2 * 8);  // (the tables are the batch's; the request's size stays as it was)
   float* mus = (float*)take((size_t)(nx + ny) * 4);
   double* parts = (double*)take((size_t)2 * (ny / 2 + 1) * 8);
   const double hx = r.grid.length[0] / nx, hy = r.grid.length[1] / ny;
@@ -816,11 +839,9 @@ bool admit(rd_batch* b, Request& q, rd_status* err) {
   d.kind = r.reaction.kind;
   d.precond = 1;
   d.mode = MODE_PDHG;
-  // tiles: the measured best for this grid size (opts.autotune), else 4-row bands, 4 columns
-  const int lg = ilog2i(std::max(nx, ny));
-  d.band_rows = std::min(b->tune_band[lg] ? b->tune_band[lg] : kBatchBandRows, ny);
+  d.band_rows = std::min(kBatchBandRows, ny);
   d.nbands = (ny + d.band_rows - 1) / d.band_rows;
-  d.col_width = std::min(b->tune_col[lg] ? b->tune_col[lg] : kBatchColWidth, nx);
+  d.col_width = std::min(kBatchColWidth, nx);
   d.ncolblk = nx / d.col_width;
   d.hx2 = 1.0 / (hx * hx);
   d.hy2 = 1.0 / (hy * hy);
@@ -858,30 +879,27 @@ bool admit(rd_batch* b, Request& q, rd_status* err) {
   d32.P[0] = p0;
   d32.P[1] = p1;
   d32.WY = wy;
-  cx<float>* twx = reinterpret_cast<cx<float>*>(tabs);
-  cx<float>* dcx = twx + nx;
-  cx<float>* twy = dcx + nx;
-  cx<float>* dcy = twy + ny;
-  d32.twx = twx;
-  d32.dcx = dcx;
-  d32.twy = twy;
-  d32.dcy = dcy;
+  d32.twx = twiddles_of(b, nx);
+  d32.dcx = rotations_of(b, nx);
+  d32.twy = twiddles_of(b, ny);
+  d32.dcy = rotations_of(b, ny);
   d32.mux = mus;
   d32.muy = mus + nx;
-  sh.d32 = d32;
-  sh.d64 = d64;
   // small grids: each inner solve in one launch (one block, or a cluster of eight)
   sh.small = b->opts.small_solve ? small_mode(nx, ny, nc, sh.key, r.bc == RD_BC_NEUMANN, b->smem_usable) : 0;
-  // tables, state, control block
-  std::vector<float> tw, dc, mu, all_t, all_mu;
-  host_tables(nx, r.bc == RD_BC_NEUMANN, hx, tw, dc, mu);
-  all_t.insert(all_t.end(), tw.begin(), tw.end());
-  all_t.insert(all_t.end(), dc.begin(), dc.end());
-  all_mu = mu;
-  host_tables(ny, r.bc == RD_BC_NEUMANN, hy, tw, dc, mu);
-  all_t.insert(all_t.end(), tw.begin(), tw.end());
-  all_t.insert(all_t.end(), dc.begin(), dc.end());
-  all_mu.insert(all_mu.end(), mu.begin(), mu.end());
+  sh.fast = !sh.small && nx >= 16 && ny >= 16;
+  if (sh.fast) {
+    int row = 0, col = 0;
+    // (at most ny / 2 blocks: the partial sums of the norm)
+    d32.blk3 = batch_lines2_plan(d32, ny / 2, &row, &col);
+    d32.P[1] = wy;
+  }
+  sh.d32 = d32;
+  sh.d64 = d64;
+  // eigenvalues, state, control block
+  std::vector<float> all_mu;
+  append_mu(b, nx, r.bc == RD_BC_NEUMANN, hx, all_mu);
+  append_mu(b, ny, r.bc == RD_BC_NEUMANN, hy, all_mu);
   Slot ctl{};
   ctl.outer.max_iter = 1 << 30;
   ctl.inner.max_iter = b->opts.max_iter;
@@ -893,14 +911,12 @@ bool admit(rd_batch* b, Request& q, rd_status* err) {
   ctl.tol_kind = r.tol_kind;
   cudaStream_t st = b->stream;
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(tabs, all_t.data(), all_t.size() * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(mus, all_mu.data(), all_mu.size() * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(u, q.u0.data(), npts * 8, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d32 + s, &sh.d32, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d64 + s, &sh.d64, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_slots + s, &ctl, sizeof(Slot), cudaMemcpyHostToDevice, st);
-  // the host vectors above are pageable: wait for the copies before they go out of scope
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  // (no wait: the copies read pageable memory, which cudaMemcpyAsync has staged when it returns)
   if (e != cudaSuccess) *err = bfail(RD_ERR_CUDA, std::string("admission: ") + cudaGetErrorString(e));
   std::lock_guard<std::mutex> lk(b->mu);
   b->stats.admitted += 1;
@@ -953,119 +969,6 @@ void retire(rd_batch* b, int s, const Slot& ctl) {
   if (!copy_error.empty()) b->worker_error = copy_error;
   b->done.push_back(res);
   b->cv.notify_all();
-}
-
-// opts.autotune: for each square grid size the arena can hold, admit one scratch Allen-Cahn slot
-// whose inner solve never stops, time graph-free launches of its three sweep kernels over 8
-// iterations (best of three) for band rows {2, 4} x column widths {2, 4}, and keep the fastest
-// per size; admission then takes the measured tiles.  Every candidate fits the launches' shared
-// memory (sized for 4-row bands and 4 columns).
-rd_status tune_batch_tiles(rd_batch* b) {
-  cudaStream_t st = b->stream;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
-    return bfail(RD_ERR_CUDA, "tile tuning: events");
-  const int g = group_of(KK_AC);
-  rd_status res = RD_OK;
-  for (int lg = 4; lg <= ilog2i(kBatchMaxSide) && res == RD_OK; ++lg) {
-    const int n = 1 << lg;
-    Request q;
-    q.req.grid.ndim = 2;
-    q.req.grid.n[0] = q.req.grid.n[1] = n;
-    q.req.grid.length[0] = q.req.grid.length[1] = 1.0;
-    q.req.bc = RD_BC_PERIODIC;
-    q.req.op = RD_OP_LAPLACIAN;
-    q.req.reaction.kind = RD_RX_ALLEN_CAHN;
-    q.req.reaction.ncomp = 1;
-    q.req.reaction.a = 0.05;
-    q.req.reaction.b = 20.0;
-    q.req.dt = 2e-3;
-    q.req.tau = q.req.sigma = 1.0;
-    q.req.tol = 1e-11;
-    q.req.tol_kind = RD_TOL_F_REL;
-    q.req.nsteps = 1;
-    q.u0.assign((size_t)n * n, 0.0);
-    rd_status err = RD_OK;
-    const int small_opt = b->opts.small_solve;
-    b->opts.small_solve = 0;  // time the sweeps, not the one-launch solve
-    const bool ok = admit(b, q, &err);
-    b->opts.small_solve = small_opt;
-    if (!ok) break;  // the arena holds no larger grid
-    int s = -1;
-    for (int k = 0; k < b->max_slots; ++k)
-      if (b->slots[k].used) s = k;
-    SlotHost& sh = b->slots[s];
-    const size_t npts = sh.npts;
-    // base state and right-hand side nonzero, d = P = 0, an inner solve that never stops
-    cudaMemsetAsync(const_cast<void*>(sh.d32.rhs), 0x3f, npts * 4, st);
-    cudaMemsetAsync(const_cast<void*>(sh.d32.base), 0x3f, npts * 4, st);
-    cudaMemsetAsync(sh.d32.X, 0, npts * 4, st);
-    cudaMemsetAsync(sh.d32.P[0], 0, npts * 4, st);
-    cudaMemsetAsync(sh.d32.P[1], 0, npts * 4, st);
-    float best = 1e30f;
-    int bb = kBatchBandRows, bc = kBatchColWidth;
-    for (int band : {2, 4})
-      for (int cw : {2, 4}) {
-        if (band > n || cw > n) continue;
-        Desc d32 = sh.d32, d64 = sh.d64;
-        d32.band_rows = d64.band_rows = band;
-        d32.nbands = d64.nbands = (n + band - 1) / band;
-        d32.col_width = d64.col_width = cw;
-        d32.ncolblk = d64.ncolblk = n / cw;
-        std::vector<int2> bands, cols;
-        for (int k = 0; k < d32.nbands; ++k) bands.push_back(make_int2(s, k));
-        for (int k = 0; k < d32.ncolblk; ++k) cols.push_back(make_int2(s, k));
-        Slot ctl{};
-        ctl.phase = PH_INNER;
-        ctl.inner.status = ST_ACTIVE;
-        ctl.inner.max_iter = 1 << 30;
-        ctl.inner.thresh = 0.0;
-        ctl.inner.stall_mul = 1 << 20;
-        cudaMemcpyAsync(b->d_d32 + s, &d32, sizeof(Desc), cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(b->d_d64 + s, &d64, sizeof(Desc), cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(b->d_slots + s, &ctl, sizeof(Slot), cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(b->d_band_items[g], bands.data(), bands.size() * sizeof(int2), cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(b->d_col_items[g], cols.data(), cols.size() * sizeof(int2), cudaMemcpyHostToDevice, st);
-        float t_best = 1e30f;
-        for (int rep = 0; rep < 3; ++rep) {
-          cudaEventRecord(e0, st);
-          for (int it = 0; it < 8; ++it) {
-            k_res_b<float, KK_AC><<<(int)bands.size(), kBatchThreads, b->smem_sweep, st>>>(b->d_d32, b->d_slots, b->d_band_items[g]);
-            k_col_b<float><<<(int)cols.size(), kBatchThreads, b->smem_sweep, st>>>(b->d_d32, b->d_slots, b->d_col_items[g]);
-            k_upd_b<float, KK_AC><<<(int)bands.size(), kBatchThreads, b->smem_sweep, st>>>(b->d_d32, b->d_slots, b->d_band_items[g]);
-          }
-          cudaEventRecord(e1, st);
-          if (cudaEventSynchronize(e1) != cudaSuccess) {
-            res = bfail(RD_ERR_CUDA, std::string("tile tuning: ") + cudaGetErrorString(cudaGetLastError()));
-            break;
-          }
-          float ms = 0.f;
-          cudaEventElapsedTime(&ms, e0, e1);
-          t_best = std::min(t_best, ms);
-        }
-        if (res != RD_OK) break;
-        if (t_best < best) {
-          best = t_best;
-          bb = band;
-          bc = cw;
-        }
-      }
-    b->tune_band[lg] = bb;
-    b->tune_col[lg] = bc;
-    // release the scratch slot
-    {
-      std::lock_guard<std::mutex> lk(b->mu);
-      b->arena.release(sh.mem, sh.mem_bytes);
-      b->stats.admitted -= 1;
-    }
-    Slot idle{};
-    cudaMemcpyAsync(b->d_slots + s, &idle, sizeof(Slot), cudaMemcpyHostToDevice, st);
-    sh = SlotHost{};
-  }
-  cudaStreamSynchronize(st);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  return res;
 }
 
 void worker_loop(rd_batch* b) {
@@ -1173,21 +1076,11 @@ rd_status rd_batch_create(rd_batch** out, size_t hbm_budget_bytes, int max_slots
     return cleanup(bfail(RD_ERR_OOM, std::string("arena: ") + cudaGetErrorString(e)));
   }
   b->arena.init(b->arena_mem, hbm_budget_bytes);
-  const int max_items = max_slots * (kBatchMaxSide / 2);
   if ((e = cudaMalloc(&b->d_d32, sizeof(Desc) * max_slots)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_d64, sizeof(Desc) * max_slots)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_slots, sizeof(Slot) * max_slots)) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_slots, sizeof(Slot) * max_slots)) != cudaSuccess)
     return cleanup(bfail(RD_ERR_OOM, cudaGetErrorString(e)));
-  for (int g = 0; g < kBatchGroups; ++g) {
-    if ((e = cudaMalloc(&b->d_band_items[g], sizeof(int2) * max_items)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_phase_items[g], sizeof(int2) * max_items)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_small_items[g][0], sizeof(int2) * max_slots)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_small_items[g][1], sizeof(int2) * max_slots)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_col_items[g], sizeof(int2) * max_items)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_items3[g], sizeof(int2) * max_slots * kBatchMaxBlk3)) != cudaSuccess)
-      return cleanup(bfail(RD_ERR_OOM, cudaGetErrorString(e)));
-  }
   cudaMemset(b->d_slots, 0, sizeof(Slot) * max_slots);
   // shared memory of the batched sweeps: the largest grid the batch accepts
   int dev = 0, optin = 0;
@@ -1197,6 +1090,12 @@ rd_status rd_batch_create(rd_batch** out, size_t hbm_budget_bytes, int max_slots
   b->smem_sweep = std::max(res_smem_bytes<float>(1, kBatchBandRows, 2, kBatchMaxSide, 1, 0, tabs),
                            std::max(lines_smem_bytes<float>((kBatchBandRows + 4) / 2, kBatchMaxSide, 0, tabs),
                                     lines_smem_bytes<float>(kBatchColWidth / 2, kBatchMaxSide, 0, tabs)));
+  if ((e = batch_lines2_allow(optin)) != cudaSuccess || (e = batch_lines3_allow(optin)) != cudaSuccess)
+    return cleanup(bfail(RD_ERR_CUDA, cudaGetErrorString(e)));
+  {
+    const rd_status ts = make_tables(b);
+    if (ts != RD_OK) return cleanup(ts);
+  }
   if ((e = batch3_allow(optin)) != cudaSuccess || (e = allow_small(optin)) != cudaSuccess)
     return cleanup(bfail(RD_ERR_CUDA, cudaGetErrorString(e)));
   b->smem_usable = optin - 1024;
@@ -1216,10 +1115,6 @@ rd_status rd_batch_create(rd_batch** out, size_t hbm_budget_bytes, int max_slots
     cudaFuncSetAttribute(k_col_b<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
   }
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cleanup(bfail(RD_ERR_CUDA, cudaGetErrorString(e)));
-  if (b->opts.autotune) {
-    const rd_status ts = tune_batch_tiles(b);
-    if (ts != RD_OK) return cleanup(ts);
-  }
   b->worker = std::thread(worker_loop, b);
   *out = b;
   return RD_OK;
@@ -1311,14 +1206,10 @@ void rd_batch_destroy(rd_batch* b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->graph) cudaGraphDestroy(b->graph);
-  for (int g = 0; g < kBatchGroups; ++g) {
-    if (b->d_band_items[g]) cudaFree(b->d_band_items[g]);
-    if (b->d_col_items[g]) cudaFree(b->d_col_items[g]);
-    if (b->d_items3[g]) cudaFree(b->d_items3[g]);
-    if (b->d_phase_items[g]) cudaFree(b->d_phase_items[g]);
-    for (int m = 0; m < 2; ++m)
-      if (b->d_small_items[g][m]) cudaFree(b->d_small_items[g][m]);
-  }
+  for (rd_batch::Lists& l : b->lists)
+    for (ItemList* it : {&l.band, &l.col, &l.small_phase, &l.small1, &l.small2, &l.line_phase, &l.line2, &l.old3, &l.line3})
+      if (it->d) cudaFree(it->d);
+  if (b->d_tables) cudaFree(b->d_tables);
   if (b->d_d32) cudaFree(b->d_d32);
   if (b->d_d64) cudaFree(b->d_d64);
   if (b->d_slots) cudaFree(b->d_slots);

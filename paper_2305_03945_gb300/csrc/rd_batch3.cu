@@ -172,10 +172,15 @@ cudaError_t allow_k(K_ kernel, int optin) {
 }
 
 template <int K>
+void phases3(const Batch3Launch& L, cudaStream_t s) {
+  k3_axpy_b<<<L.nitems, 256, 0, s>>>(L.d64s, L.slots, L.items);
+  k3_step_b<K><<<L.nitems, 256, 0, s>>>(L.d64s, L.slots, L.items);
+}
+
+template <int K>
 void group3(const Batch3Launch& L, cudaStream_t s) {
   const int n = L.nitems;
-  k3_axpy_b<<<n, 256, 0, s>>>(L.d64s, L.slots, L.items);
-  k3_step_b<K><<<n, 256, 0, s>>>(L.d64s, L.slots, L.items);
+  phases3<K>(L, s);
   k3_res_b<K><<<n, 256, 0, s>>>(L.d32s, L.slots, L.items);
   k3_lines_b<0, L3_FWD><<<n, L.thr[0], L.smem[0], s>>>(L.d32s, L.slots, L.items);
   k3_lines_b<1, L3_FWD><<<n, L.thr[1], L.smem[1], s>>>(L.d32s, L.slots, L.items);
@@ -186,6 +191,19 @@ void group3(const Batch3Launch& L, cudaStream_t s) {
 }
 
 }  // namespace
+
+cudaError_t batch3_launch_phases(int key, const Batch3Launch& L, cudaStream_t s) {
+  if (L.nitems == 0) return cudaSuccess;
+  switch (key) {
+    case KK_NONE_LAP: phases3<KK_NONE_LAP>(L, s); break;
+    case KK_AC: phases3<KK_AC>(L, s); break;
+    case KK_CH_IMPL: phases3<KK_CH_IMPL>(L, s); break;
+    case KK_CH_SPLIT: phases3<KK_CH_SPLIT>(L, s); break;
+    case KK_NONE_BIH: phases3<KK_NONE_BIH>(L, s); break;
+    default: return cudaErrorNotSupported;
+  }
+  return cudaGetLastError();
+}
 
 cudaError_t batch3_launch_group(int key, const Batch3Launch& L, cudaStream_t s) {
   if (L.nitems == 0) return cudaSuccess;

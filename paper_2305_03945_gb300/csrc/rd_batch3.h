@@ -21,6 +21,8 @@ struct Batch3Launch {
   int smem[3];
 };
 
+// The step phases alone (u += d; step set-up, FP64 residual and outer decision).
+cudaError_t batch3_launch_phases(int key, const Batch3Launch& L, cudaStream_t s);
 cudaError_t batch3_launch_group(int key, const Batch3Launch& L, cudaStream_t s);
 // Raise the dynamic shared-memory limit of the batched 3-D transform passes.
 cudaError_t batch3_allow(int optin);

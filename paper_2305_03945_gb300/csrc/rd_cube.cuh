@@ -66,15 +66,14 @@ struct Pt4z {
 // ---------------------------------------------------------------------------------------
 // k3_rowres
 // ---------------------------------------------------------------------------------------
+// The lines of group `blk`; the squares of the thread's residuals are added to acc_out.
 template <class T, int K, int LOGN, int V>
-__device__ __forceinline__ void rowres3_body(const Desc& d, State* __restrict__ st, Slot* slot, int blk, int nblk,
-                                             unsigned char* smem_raw) {
+__device__ __forceinline__ void rowres3_body(const Desc& d, int blk, unsigned char* smem_raw, T& acc_out) {
   using F = Rf<LOGN, V>;
   constexpr int N = F::N;
   constexpr int H = KT<K>::H;
   constexpr bool DC = sizeof(T) == 4;
   constexpr bool BASE = DC && KT<K>::nonlinear;
-  __shared__ double red[32];
   const int lline = threadIdx.x / F::TPL, t = threadIdx.x % F::TPL;
   const int lines = d.nz * (d.ny >> 1);
   const int gl = blk * (blockDim.x / F::TPL) + lline;
@@ -121,8 +120,19 @@ __device__ __forceinline__ void rowres3_body(const Desc& d, State* __restrict__ 
   auto sync = [lline] { line_sync<F::TPL>(lline); };
   sync();
   row_forward<T, LOGN, V>(d, line, static_cast<T*>(d.WY) + o, t, live, sync);
-  const double s = block_sum(live ? (double)acc : 0.0, red);
-  if (threadIdx.x == 0) d.partials[blk] = s;
+  if (live) acc_out += acc;
+}
+
+// Partial norm of block `blk` of `nblk`, stopping decision in the last one.
+__device__ __forceinline__ void rowres_finish(const Desc& d, State* __restrict__ st, Slot* slot, int blk, int nblk, float a0,
+                                              float a1) {
+  __shared__ double red[32];
+  const double s0 = block_sum((double)a0, red);
+  const double s1 = d.ncomp == 2 ? block_sum((double)a1, red) : 0.0;
+  if (threadIdx.x == 0) {
+    d.partials[blk] = s0;
+    if (d.ncomp == 2) d.partials[nblk + blk] = s1;
+  }
   if (last_block(st, nblk)) finalize_measure(d, st, red, slot, nblk);
 }
 
@@ -131,21 +141,25 @@ __global__ void __launch_bounds__(256) k3_rowres(const __grid_constant__ Desc d,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
   if (!sweep_active(st, nullptr)) return;
-  rowres3_body<T, K, LOGN, V>(d, st, nullptr, blockIdx.x, gridDim.x, smem_raw);
+  T acc = T(0);
+  rowres3_body<T, K, LOGN, V>(d, blockIdx.x, smem_raw, acc);
+  rowres_finish(d, st, nullptr, blockIdx.x, gridDim.x, acc, 0.f);
 }
 
 // ---------------------------------------------------------------------------------------
-// k3_axis: transforms along y (AX = 1) and z (AX = 2), `nl` adjacent column pairs per block
+// k3_axis: transforms along y (AX = 1) and z (AX = 2), `nl` adjacent column pairs per block; `sync` is a
+// barrier of the nl TPL threads.  Scalar 3-D grids; 2-D grids (nz <= 1, AX = 1) with either number of
+// components.
 // ---------------------------------------------------------------------------------------
-template <class T, int AX, int MODE, int LOGN, int V>
-__device__ __forceinline__ void axis3_body(const Desc& d, int nl, int blk, unsigned char* smem_raw) {
+template <class T, int AX, int MODE, int LOGN, int V, class Sync>
+__device__ __forceinline__ void axis3_body(const Desc& d, int nl, int blk, unsigned char* smem_raw, Sync sync) {
   using F = Rf<LOGN, V>;
   using P1 = Pass<T, LOGN, V, true, 1>;
   constexpr int N = F::N;
   const int hx = d.nx >> 1;
   const int m = threadIdx.x % nl, t = threadIdx.x / nl;
   const int ntx = hx / nl;
-  const int third = blk / ntx;                    // z of a y line, y of a z line
+  const int third = blk / ntx;                    // z of a y line, y of a z line (2-D: the component)
   const int col = (blk - third * ntx) * nl + m;   // pair of columns
   const size_t plane = (size_t)hx * d.ny;
   const size_t rs = AX == 1 ? hx : plane;         // pairs between the elements of a line
@@ -154,7 +168,6 @@ __device__ __forceinline__ void axis3_body(const Desc& d, int nl, int blk, unsig
   const cx<T>* tw = static_cast<const cx<T>*>(AX == 1 ? d.twy : d.twz);
   const cx<T>* dc = static_cast<const cx<T>*>(AX == 1 ? d.dcy : d.dcz);
   cx<T>* buf = reinterpret_cast<cx<T>*>(smem_raw) + m;
-  auto sync = [] { __syncthreads(); };
   cx<T> v[V];
   // frequency of paired value i and its partner (the self-paired 0 and N/2 in thread 0)
   auto freq = [&](int i) { return rf_freq<V>(N, t, i); };
@@ -170,9 +183,9 @@ __device__ __forceinline__ void axis3_body(const Desc& d, int nl, int blk, unsig
   if constexpr (MODE == L3_FSI) {
     const T* mux = static_cast<const T*>(d.mux);
     const T* muo = static_cast<const T*>(AX == 1 ? d.muz : d.muy);
-    const T mo = __ldg(muo + third);
+    const T mo = d.nz > 1 ? __ldg(muo + third) : T(0);
     scale_pairs<T, N, V>(v, t, per,
-                         SymMu<T>{Symbol<T>(d, 0), static_cast<const T*>(AX == 1 ? d.muy : d.muz),
+                         SymMu<T>{Symbol<T>(d, d.nz > 1 ? 0 : third), static_cast<const T*>(AX == 1 ? d.muy : d.muz),
                                   __ldg(mux + 2 * col) + mo, __ldg(mux + 2 * col + 1) + mo},
                          dc);
   }
@@ -234,7 +247,7 @@ __global__ void __launch_bounds__(BandThreads<T, V>::value) k3_axis(const __grid
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
   if (st && !sweep_active(st, nullptr)) return;  // st = nullptr: the preconditioner alone
-  axis3_body<T, AX, MODE, LOGN, V>(d, nl, blockIdx.x, smem_raw);
+  axis3_body<T, AX, MODE, LOGN, V>(d, nl, blockIdx.x, smem_raw, [] { __syncthreads(); });
 }
 
 // ---------------------------------------------------------------------------------------

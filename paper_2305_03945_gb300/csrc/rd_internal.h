@@ -86,6 +86,7 @@ struct Desc {
   int blk3;
   int lw3[3];
   int thr3[3];       // threads per block of the transform pass of each axis
+  int fastb;         // batch: 1 when the slot runs the kernels of rd_batch_lines.cuh (blk3 blocks each)
   int pf3;           // 1: the long x inverse pass prefetches its P rows into shared memory
 };
 
