@@ -15,6 +15,8 @@
 // k_rowfwd is the forward row transform alone (preconditioner-only solve).
 #pragma once
 
+#include <cuda.h>
+
 #include <type_traits>
 
 #include "rd_fft.cuh"
@@ -179,6 +181,105 @@ __global__ void __launch_bounds__(ColThreads<T, LOGN, V>::value, ColThreads<T, L
   pdl_wait();
   if (st && !sweep_active(st, nullptr)) return;
   fcol_body<T, LOGN, V, PER>(d, blockIdx.x, smem_raw);
+}
+
+// ---------------------------------------------------------------------------------------
+// k_fcol_tma: k_fcol<float> at V = 16 on lines of 2048 points and more, whose tile of narrow row segments
+// TMA moves between global and shared memory: by threads, a warp's load or store of such a tile is 8 or 16
+// separate requests, and their issue was the kernel's first stall (lg_throttle).  Measured, k_fcol ->
+// k_fcol_tma: 2048^2 x 2 (32-byte segments) 50 -> 37 us, 1.8 TB/s; 8192^2 (16-byte segments) 578 -> 394 us,
+// 1.4 TB/s.  On 1024^2, a block or two per SM, it was slower (step 0.749 -> 0.785 ms): the tile's way
+// through shared memory has nothing to hide behind.
+// ---------------------------------------------------------------------------------------
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// Waits for phase 0 of a transaction barrier, with a bound (false: it ran out).
+__device__ __forceinline__ bool mbar_wait0(unsigned bar) {
+  for (int i = 0; i < (1 << 22); ++i) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+constexpr int kTmaRows = 256;  // rows of one TMA box (the largest)
+
+template <int LOGN>
+struct TmaCol {
+  static constexpr int threads = LOGN >= 12 ? 1024 : 512;
+  static constexpr int blocks = LOGN >= 12 ? 1 : 2;
+};
+
+template <int LOGN, bool PER>
+__global__ void __launch_bounds__(TmaCol<LOGN>::threads, TmaCol<LOGN>::blocks)
+    k_fcol_tma(const __grid_constant__ Desc d, State* __restrict__ st, const __grid_constant__ CUtensorMap map) {
+  constexpr int V = 16;
+  using F = Rf<LOGN, V>;
+  using P1 = Pass<float, LOGN, V, true, 1>;
+  constexpr int N = F::N;
+  extern __shared__ __align__(128) unsigned char smem_tma[];
+  __shared__ __align__(8) unsigned long long bar;
+  pdl_wait();
+  if (!sweep_active(st, nullptr)) return;
+  const int nl = d.col_width >> 1, lnl = ilog2i(nl);
+  const int m = threadIdx.x & (nl - 1), t = threadIdx.x >> lnl;
+  const int c = blockIdx.x / d.ncolblk, x0 = (blockIdx.x - c * d.ncolblk) * d.col_width;
+  const int col = x0 + 2 * m;
+  const unsigned mb = smem_u32(&bar), box = kTmaRows * d.col_width * 4;
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"((unsigned)(N / kTmaRows) * box) : "memory");
+    for (int k = 0; k < N / kTmaRows; ++k)
+      asm volatile(
+          "cp.async.bulk.tensor.2d.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+              smem_u32(smem_tma) + k * box),
+          "l"(&map), "r"(x0), "r"(c * N + k * kTmaRows), "r"(mb)
+          : "memory");
+  }
+  __syncthreads();  // the barrier is initialised
+  cx<float>* buf = reinterpret_cast<cx<float>*>(smem_tma) + m;
+  if (!mbar_wait0(mb)) {  // cannot happen while the memory system works; the tile stays as it was
+    if (threadIdx.x == 0) st->status = ST_DIVERGED;
+    mbar_wait0(mb);
+    return;
+  }
+  cx<float> v[V];
+#pragma unroll
+  for (int e = 0; e < V; ++e) {
+    const int n = P1::natural(t, e);
+    v[e] = buf[(PER ? n : mk_perm(n, N)) * nl];
+  }
+  auto sync = [] { __syncthreads(); };
+  sync();
+  const cx<float>* tw = static_cast<const cx<float>*>(d.twy);
+  rf_forward<float, LOGN, V, true>(v, buf, nl, tw, t, sync);
+  const float* mux = static_cast<const float*>(d.mux);
+  scale_pairs<float, N, V>(
+      v, t, PER, SymMu<float>{Symbol<float>(d, c), static_cast<const float*>(d.muy), __ldg(mux + col), __ldg(mux + col + 1)},
+      static_cast<const cx<float>*>(d.dcy));
+  rf_inverse<float, LOGN, V, true>(v, buf, nl, tw, t, sync);
+  sync();
+#pragma unroll
+  for (int e = 0; e < V; ++e) {
+    const int n = P1::natural(t, e);
+    buf[(PER ? n : mk_perm(n, N)) * nl] = v[e];
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < N / kTmaRows; ++k)
+      asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(&map), "r"(x0),
+                   "r"(c * N + k * kTmaRows), "r"(smem_u32(smem_tma) + k * box)
+                   : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -454,21 +555,22 @@ template <int K>
 __host__ __device__ constexpr int ncomp_of() { return KT<K>::two ? 2 : 1; }
 
 // Shared-memory bytes of a k_primal block: the band's rows of U with H halo rows, then reused by
-// the line buffers of the forward transform.
+// the line buffers of the forward transform; and in front the table of row offsets.
 template <class T>
 __host__ __device__ inline int primal_smem_bytes(int nc, int rows, int H, int nx, int line_len, int line_bufs) {
   const int u = nc * (rows + 2 * H) * nx * (int)sizeof(T);
   const int l = line_bufs * line_len * (int)sizeof(cx<T>);
-  return u > l ? u : l;
+  return (u > l ? u : l) + (rows + 2 * H) * (2 * H + 1) * (int)sizeof(int);
 }
 
-// Threads of a k_primal block at most, and the blocks an SM shall hold (the register cap): FP32 lines of
-// 4096 and 8192 points take 1024 threads; FP32 five-point kinds at V = 16 two blocks of 512 (64
-// registers, up to 100 bytes spilled for two species); the thirteen-point kinds would spill more.
+// Threads of a k_primal block at most, and the blocks an SM shall hold (the register cap).  FP32 lines of
+// 2048 points and more: 1024 threads, 64 registers (two species spill 100 bytes): two blocks of four rows
+// or one of eight per SM; FP32 five-point kinds at V = 16 on shorter lines: two blocks of 512.
 template <class T, int K, int LOGN, int V>
 struct PrimalBlock {
-  static constexpr int threads = sizeof(T) == 4 && LOGN >= 12 ? 1024 : BandThreads<T, V>::value;
-  static constexpr int blocks = sizeof(T) == 4 && V == 16 && LOGN < 12 && !KT<K>::biharm ? 2 : 1;
+  static constexpr bool wide = sizeof(T) == 4 && V == 16 && LOGN >= 11;
+  static constexpr int threads = wide ? 1024 : BandThreads<T, V>::value;
+  static constexpr int blocks = sizeof(T) == 4 && V == 16 && !wide && !KT<K>::biharm ? 2 : 1;
 };
 
 template <class T, int K, int LOGN, int V>
@@ -490,7 +592,16 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
   const int y0 = band * B;
   const int rows = min(B, ny - y0);
   const int srows = rows + 2 * H;
-  T* us = reinterpret_cast<T*>(smem_raw);
+  // offsets of the rows the stencils of every staged row read, boundary-mapped (a row beyond a wall is
+  // updated exactly as the row it maps to, by that row's neighbours); mapped per group of four points they
+  // cost 7% of the kernel's instructions (steps: 1024 x 128 805 -> 782 us, 512^2 716 -> 705 us)
+  int* roff = reinterpret_cast<int*>(smem_raw);
+  const int tab = (srows * (2 * H + 1) + 3) / 4 * 4;
+  T* us = reinterpret_cast<T*>(smem_raw + tab * sizeof(int));
+  for (int k = tid; k < srows * (2 * H + 1); k += nt) {
+    const int r = k / (2 * H + 1), di = k - r * (2 * H + 1) - H;
+    roff[k] = bcmap(bcmap(y0 + r - H, ny, bc) + di, ny, bc) << LOGN;
+  }
   T* X = static_cast<T*>(d.X);
   T* Hb = static_cast<T*>(d.halo) + (size_t)band * NC * 2 * H * N;
   const T* Bs = static_cast<const T*>(d.base);
@@ -500,14 +611,17 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
   // 1. U_{n+1} on the band and its halo rows: band rows in place in X, halo rows in this block's
   //    own copy (rows that other blocks update), all rows staged in shared memory.  `first`: U_0.
   const T tu = T(d.tau_u);
+  __syncthreads();
   for (int g = tid; g < (srows << LV); g += nt) {
     const int r = (g >> LV) - H, j0 = (g & ((1 << LV) - 1)) * 4;
     const bool own = r >= 0 && r < rows;
-    const int row = bcmap(y0 + r, ny, bc);
+    const int* ro = roff + (r + H) * (2 * H + 1);
+    const int at = ro[H] + j0;
     T* u[2];
     const int slot = r < 0 ? r + H : r - rows + H;
-    u[0] = own || first ? X + (size_t)row * N + j0 : Hb + (size_t)slot * N + j0;
-    u[1] = own || first ? u[0] + plane : Hb + (size_t)(2 * H + slot) * N + j0;
+    const int hat = (slot << LOGN) + j0;
+    u[0] = own || first ? X + at : Hb + hat;
+    u[1] = own || first ? u[0] + plane : Hb + (2 * H << LOGN) + hat;
     T x[2][4];
 #pragma unroll
     for (int c = 0; c < NC; ++c) ld4(u[c], x[c]);
@@ -515,11 +629,11 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
       T s[2][4] = {};
       if constexpr (BASE)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) ld4(Bs + c * plane + (size_t)row * N + j0, s[c]);
+        for (int c = 0; c < NC; ++c) ld4(Bs + c * plane + at, s[c]);
       Patch<T, H> p[NC];
       const T* rp[2 * H + 1];
 #pragma unroll
-      for (int di = -H; di <= H; ++di) rp[H + di] = Pt + (size_t)bcmap(row + di, ny, bc) * N;
+      for (int di = 0; di <= 2 * H; ++di) rp[di] = Pt + ro[di];
       p[0].load(rp, j0, N, per);
       if constexpr (NC == 2) {
 #pragma unroll
@@ -535,13 +649,13 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
       }
     }
     if (!own) {
-      u[0] = Hb + (size_t)slot * N + j0;
-      u[1] = Hb + (size_t)(2 * H + slot) * N + j0;
+      u[0] = Hb + hat;
+      u[1] = Hb + (2 * H << LOGN) + hat;
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       if (!first || !own) st4(u[c], x[c]);
-      st4(us + (size_t)(c * srows + r + H) * N + j0, x[c]);
+      st4(us + ((c * srows + r + H) << LOGN) + j0, x[c]);
     }
   }
   __syncthreads();
@@ -559,16 +673,17 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
       const int r = 2 * (g >> LV), j0 = (g & ((1 << LV) - 1)) * 4;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int row = y0 + r + h;
+        const int* ro = roff + (r + h + H) * (2 * H + 1);
+        const int at = ro[H] + j0;
         T rr[2][4];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) ld4(static_cast<const T*>(d.rhs) + c * plane + (size_t)row * N + j0, rr[c]);
+        for (int c = 0; c < NC; ++c) ld4(static_cast<const T*>(d.rhs) + c * plane + at, rr[c]);
         Patch<T, H> x[NC];
         const T* rp[2 * H + 1];
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
 #pragma unroll
-          for (int di = -H; di <= H; ++di) rp[H + di] = us + (size_t)(c * srows + r + h + H + di) * N;
+          for (int di = -H; di <= H; ++di) rp[H + di] = us + ((c * srows + r + h + H + di) << LOGN);
           x[c].load(rp, j0, N, per);
         }
         auto points = [&](const auto& b0, const auto& b1) {
@@ -587,13 +702,13 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
           Patch<T, 1> b;
           const T* bp[3];
 #pragma unroll
-          for (int di = -1; di <= 1; ++di) bp[1 + di] = Bs + (size_t)bcmap(row + di, ny, bc) * N;
+          for (int di = -1; di <= 1; ++di) bp[1 + di] = Bs + ro[H + di];
           b.load(bp, j0, N, per);
           points(b, b);
         } else if constexpr (BASE) {
           Pt4<T> b[NC];
 #pragma unroll
-          for (int c = 0; c < NC; ++c) ld4(Bs + c * plane + (size_t)row * N + j0, b[c].v);
+          for (int c = 0; c < NC; ++c) ld4(Bs + c * plane + at, b[c].v);
           points(b[0], b[NC - 1]);
         } else {
           points(x[0], x[NC - 1]);
@@ -602,7 +717,7 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
     }
   }
   __syncthreads();
-  cx<T>* lines = reinterpret_cast<cx<T>*>(smem_raw);
+  cx<T>* lines = reinterpret_cast<cx<T>*>(us);
   constexpr int LEN = Lay<T, LOGN, V, false>::len;
   const int hr = rows >> 1;
 #pragma unroll

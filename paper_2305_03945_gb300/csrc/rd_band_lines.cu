@@ -26,6 +26,11 @@ cudaError_t launch_fcol(const Desc& d, State* st, const LaunchCfg& c, cudaStream
   if (sizeof(T) == 8 && !d.scale) return cudaErrorInvalidValue;  // the handle holds no symbol table
   return by_len<T>(d.logny, c.vcol, [&](auto l, auto v) {
     constexpr int L = decltype(l)::value, V = decltype(v)::value;
+    if constexpr (sizeof(T) == 4 && V == 16 && L >= 11) {
+      if (c.tmap && !pc)
+        return launch_pdl(d.bc == BC_PERIODIC ? k_fcol_tma<L, true> : k_fcol_tma<L, false>, c.grid_cols, c.thr_fcol, c.smem_fcol,
+                          s, d, st, *static_cast<const CUtensorMap*>(c.tmap));
+    }
     return launch_pdl(d.bc == BC_PERIODIC ? k_fcol<T, L, V, true> : k_fcol<T, L, V, false>, c.grid_cols, c.thr_fcol,
                       c.smem_fcol, s, d, pc ? nullptr : st);
   });
@@ -35,6 +40,27 @@ cudaError_t launch_symbol(const Desc& d, double* table, cudaStream_t s) {
   const size_t n = (size_t)d.ncomp * d.nx * d.ny;
   k_symbol<<<(unsigned)std::min<size_t>((n + 255) / 256, 8 * 152), 256, 0, s>>>(d, table);
   return cudaGetLastError();
+}
+
+bool make_col_map(const Desc& d, const LaunchCfg& c, void* map) {
+  if (!c.fast_col || c.vcol != 16 || d.ny < 2048 || d.col_width < 4) return false;
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const cuuint64_t dims[2] = {(cuuint64_t)d.nx, (cuuint64_t)d.ncomp * d.ny};
+  const cuuint64_t strides[1] = {(cuuint64_t)d.nx * sizeof(float)};
+  const cuuint32_t box[2] = {(cuuint32_t)d.col_width, (cuuint32_t)kTmaRows};
+  const cuuint32_t one[2] = {1, 1};
+  return reinterpret_cast<Encode>(fn)(static_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, d.WY, dims, strides, box,
+                                      one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <class T>
@@ -111,6 +137,11 @@ cudaError_t allow_band(const Desc& d, const LaunchCfg& c, int optin, bool primal
   if (c.transform && has_len<T>(d.logny, c.vcol))
     e = by_len<T>(d.logny, c.vcol, [&](auto l, auto v) {
       constexpr int L = decltype(l)::value, V = decltype(v)::value;
+      if constexpr (sizeof(T) == 4 && V == 16 && L >= 11) {
+        const cudaError_t r =
+            d.bc == BC_PERIODIC ? allow_smem_k(k_fcol_tma<L, true>, optin) : allow_smem_k(k_fcol_tma<L, false>, optin);
+        if (r != cudaSuccess) return r;
+      }
       return d.bc == BC_PERIODIC ? allow_smem_k(k_fcol<T, L, V, true>, optin) : allow_smem_k(k_fcol<T, L, V, false>, optin);
     });
   if (c.fast_row && e == cudaSuccess)
@@ -152,7 +183,7 @@ void plan_band(const Desc& d, int H, int smem_limit, LaunchCfg& c) {
   }
   if (has_len<T>(d.lognx, c.vrow)) {
     const int tpl = d.nx / c.vrow, len = line_len<T, false>(d.lognx, c.vrow);
-    const int cap = d.nx > 2048 && sizeof(T) == 4 ? 1024 : band_threads_max(sizeof(T), c.vrow);  // k_primal
+    const int cap = d.nx >= 2048 && sizeof(T) == 4 && c.vrow == 16 ? 1024 : band_threads_max(sizeof(T), c.vrow);  // k_primal
     // k_dual: blocks of one warp or one line at least, of up to 256 threads once the lines give
     // two blocks per SM
     const int lines = nc * (d.ny / 2);

@@ -1,5 +1,6 @@
 // C ABI of the GB300 PDHG solver: handle lifecycle, workspace and table set-up, CUDA-graph
 // capture of the PDHG iteration, and the step / solve drivers (Algorithm 1 of arxiv 2305.03945).
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -235,6 +236,7 @@ struct rd_pdhg {
   int nz = 1;       // 3-D grids: points along z (1 on a 2-D grid)
   int nd3 = 0;      // 1: a 3-D grid, or a 2-D grid on the line kernels (rd_3d.cu)
   int long2d = 0;   // 1: a 2-D side beyond 2048 (FP32) / 4096 (FP64) points
+  CUtensorMap colmap{};  // k_fcol_tma's view of the FP32 transform buffer
   Cube3 cube{};     // FP32 3-D grids on the kernels of rd_cube.cuh
   int small = 0;    // every FP32 inner solve in one launch (rd_small.cu): 1 one block, 2 a cluster
   double hz = 0;
@@ -1202,6 +1204,7 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
       RD_TRY(h->dc ? autotune_plan<float>(h, H, transform, stage_base, usable, fused)
                    : autotune_plan<double>(h, H, transform, stage_base, usable, fused));
     }
+    if (h->dc && fused && make_col_map(d, c, &h->colmap)) c.tmap = &h->colmap;
     if (fused) RD_TRY(h->dc ? plan_fused<float>(h, H) : plan_fused<double>(h, H));
     RD_CUDA(cudaMemcpy(h->d_desc, h->h_desc, 3 * sizeof(Desc), cudaMemcpyHostToDevice));
   }

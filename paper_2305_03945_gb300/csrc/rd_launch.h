@@ -20,6 +20,7 @@ struct LaunchCfg {
   int fast_row;      // k_rowfwd, k_dual, k_primal
   int vcol, vrow;    // values of a line per thread (rd_fft.cuh): 16 or 4
   int thr_fcol, smem_fcol;
+  const void* tmap;  // tensor map of WY for k_fcol_tma (make_col_map); nullptr: k_fcol
   int thr_dual, smem_dual;      // k_rowfwd, k_dual
   int thr_primal, smem_primal;
 };
@@ -46,6 +47,9 @@ cudaError_t launch_col(const Desc& d, State* st, const LaunchCfg& c, cudaStream_
 // plan (d, c) launches, and the planning rule of their launch shapes.
 template <class T>
 cudaError_t launch_fcol(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc);
+// Encodes the tensor map of d.WY for tiles of d.col_width columns into *map (a CUtensorMap) where
+// k_fcol_tma can run them (FP32 lines of 2048 points and more); false elsewhere.
+bool make_col_map(const Desc& d, const LaunchCfg& c, void* map);
 // The FP64 symbol table k_fcol<double> reads through Desc::scale ([ncomp][ny][nx]).
 cudaError_t launch_symbol(const Desc& d, double* table, cudaStream_t s);
 template <class T>

@@ -80,3 +80,21 @@ def test_step_matches_oracle_at_the_edges(kind, bc, ny, nx, rows, precision):
     U, _ = O.pdhg_step(pb, uk)
     assert info["status"] == 0, info
     assert np.linalg.norm(out.cpu().numpy() - U) <= 1e-9 * np.linalg.norm(U)
+
+
+@pytest.mark.parametrize("kind,bc,ny,nx", [("allen_cahn", "neumann", 2048, 512), ("gray_scott", "neumann", 2048, 512),
+                                           ("ch_split", "periodic", 2048, 1024), ("allen_cahn", "neumann", 4096, 256),
+                                           ("allen_cahn", "neumann", 8192, 128), ("ch_split", "periodic", 4096, 16)])
+def test_columns_moved_by_tma(kind, bc, ny, nx):
+    """The FP32 column solve on lines of 2048 points and more (k_fcol_tma): both boundaries, one and two
+    components, the narrowest grid its tiles cover."""
+    from paper_2305_03945_gb300 import rd
+    pb = _pb(kind, bc, ny, nx).replace(ly=4.0, lx=4.0 * nx / ny)
+    uk = _state(pb, 6)
+    with rd.Solver(pb, precision="fp32_dc") as s:
+        u = torch.from_numpy(uk).cuda()
+        out = torch.empty_like(u)
+        info = s.step(u, out)
+    U, _ = O.pdhg_step(pb, uk)
+    assert info["status"] == 0, info
+    assert np.linalg.norm(out.cpu().numpy() - U) <= 1e-9 * np.linalg.norm(U)
