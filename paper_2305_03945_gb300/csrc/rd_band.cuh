@@ -195,7 +195,7 @@ __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)_
 
 // Waits for phase 0 of a transaction barrier, with a bound (false: it ran out).
 __device__ __forceinline__ bool mbar_wait0(unsigned bar) {
-  for (int i = 0; i < (1 << 22); ++i) {
+  for (int i = 0; i < (1 << 20); ++i) {
     unsigned done;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
