@@ -146,7 +146,10 @@ def kernel_bytes(pb, precision, line_kernels=False, fused=False):
         # kernels have three transform passes (x, y with the scaling, x with the dual update).
         base3 = 1 if precision == "fp32_dc" else 0
         passes = 12 if getattr(pb, "nz", 1) > 1 else 8
-        return {"k3_res": (3 + base3) * es * npts, "k3_lines": passes * es * npts, "k3_upd": (3 + base3) * es * npts}
+        # FP32 3-D grids with sides of 16 to 1024 points (cube_kernels): the residual writes the x
+        # spectrum; the y, z, y passes read and write it, k_dual reads Y and P and writes P and P~
+        return {"k3_res": (3 + base3) * es * npts, "k3_lines": passes * es * npts, "k3_upd": (3 + base3) * es * npts,
+                "k3_rowres": (3 + base3) * es * npts, "k3_axis+k_dual": 10 * es * npts, "k3_primal": (3 + base3) * es * npts}
     if pb.kind == "fch":
         # sixth-order equation (FP64 stencil chains): residual mu, A mu, F = 2 + 3 + 4 touches;
         # preconditioner-only transforms 2 + 2 + 2; update dual, Lap P~, A Lap P~, U = 4 + 2 + 3 + 6
@@ -161,7 +164,12 @@ def kernel_bytes(pb, precision, line_kernels=False, fused=False):
             "k_dual+k_primal": (9 + base) * es * npts, "k_small": 5 * es * npts, "k_small_cluster": 5 * es * npts}
 
 
-def kernel_names(pb, st):
+def cube_kernels(pb, precision):
+    """Whether a 3-D problem runs the kernels of rd_cube.cuh."""
+    return precision == "fp32_dc" and pb.nz > 1 and all(16 <= n <= 1024 for n in (pb.nx, pb.ny, pb.nz))
+
+
+def kernel_names(pb, st, precision):
     """Names of the kernels behind rd_stats.kernel_ms[0..2] for this problem and handle."""
     if st.get("small_solve"):
         return ("k_small_cluster" if st["small_solve"] == 2 else "k_small",)
@@ -169,17 +177,24 @@ def kernel_names(pb, st):
         return ("fch_residual", "precond", "fch_update")
     if st.get("fused_update"):
         return ("k_primal_first", "k_fcol", "k_dual+k_primal")
+    if cube_kernels(pb, precision):
+        return ("k3_rowres", "k3_axis+k_dual", "k3_primal")
     if getattr(pb, "nz", 1) > 1 or st.get("line_kernels"):
         return ("k3_res", "k3_lines", "k3_upd")
     return ("k_res", "k_col", "k_upd")
 
 
 # the files that define each profiled kernel: a traffic figure stays valid while they are unchanged
-SWEEP_SOURCES = ("rd_band.cuh", "rd_fft.cuh", "rd_band_lines.cu", "rd_sweep.cuh", "rd_device.cuh", "rd_internal.h", "rd_launch.h", "rd_sweep_col.cu",
+SWEEP_SOURCES = ("rd_sweep.cuh", "rd_device.cuh", "rd_internal.h", "rd_launch.h", "rd_sweep_col.cu",
                  "rd_sweep_f32_lap.cu", "rd_sweep_f32_bih.cu", "rd_sweep_f64_lap.cu", "rd_sweep_f64_bih.cu")
+BAND_SOURCES = ("rd_band.cuh", "rd_fft.cuh", "rd_band_lines.cu", "rd_sweep.cuh", "rd_device.cuh", "rd_internal.h",
+                "rd_launch.h")
 SOURCES_3D = ("rd_3d.cuh", "rd_3d.cu", "rd_sweep.cuh", "rd_device.cuh", "rd_internal.h", "rd_launch3.h")
 KERNEL_SOURCES = {"k_res": SWEEP_SOURCES, "k_col": SWEEP_SOURCES, "k_upd": SWEEP_SOURCES,
-                  "k_updres": SWEEP_SOURCES + ("rd_fused_lap.cu", "rd_fused_bih.cu"),
+                  "k_primal_first": BAND_SOURCES, "k_fcol": BAND_SOURCES, "k_dual+k_primal": BAND_SOURCES,
+                  "k3_rowres": BAND_SOURCES + ("rd_cube.cuh", "rd_cube.cu", "rd_3d.cuh"),
+                  "k3_axis+k_dual": BAND_SOURCES + ("rd_cube.cuh", "rd_cube.cu", "rd_3d.cuh"),
+                  "k3_primal": BAND_SOURCES + ("rd_cube.cuh", "rd_cube.cu", "rd_3d.cuh"),
                   "k_resid64": SWEEP_SOURCES + ("rd_kernels.cu",),
                   "k3_res": SOURCES_3D, "k3_lines": SOURCES_3D, "k3_upd": SOURCES_3D}
 
@@ -426,7 +441,7 @@ def run_ours(args, rank, world, local_rank):
     # per-kernel roofline from the live CUDA-event samples
     peak, peak_kind = load_peaks()
     kb = kernel_bytes(pb, args.precision, st.get("line_kernels", 0), st.get("fused_update", 0))
-    names = kernel_names(pb, st)
+    names = kernel_names(pb, st, args.precision)
     per = {}
     for i, nm in enumerate(names):
         n = st["kernel_samples"][i]
@@ -490,7 +505,7 @@ def run_ours(args, rank, world, local_rank):
         st64 = sv64.stats()
         kb64 = kernel_bytes(pb, "fp64", st64.get("line_kernels", 0), st64.get("fused_update", 0))
         per64 = {}
-        for i, nm in enumerate(kernel_names(pb, st64)):
+        for i, nm in enumerate(kernel_names(pb, st64, "fp64")):
             n = st64["kernel_samples"][i]
             if n:
                 a = st64["kernel_ms"][i] / n
