@@ -5,12 +5,13 @@
 // phase drives FP64 defect correction and the time-step loop on the device:
 //   BEGIN  -> build the step's rhs from U^k and the outer threshold (k_step_b)
 //   RESID  -> r = F(u) in FP64, outer stopping rule, arm the FP32 inner solve (k_step_b)
-//   INNER  -> FP32 G-prox PDHG iterations on the correction equation (k_res_b, k_col_b,
-//             k_upd_b), returning to AXPY when the inner solve stops
+//   INNER  -> FP32 G-prox PDHG iterations on the correction equation (the line kernels of
+//             rd_batch_lines.cuh; k_res_b, k_col_b, k_upd_b with a side below 16 points; one launch
+//             per inner solve for small grids), returning to AXPY when the inner solve stops
 //   AXPY   -> u += d in FP64 (k_axpy_b)
 //   DONE / FAILED after the last step or on divergence.
-// One CUDA graph holds graph_k iterations of [axpy, step, res, col, upd] for each equation kind
-// present; every launch covers all slots of that kind through a work list of (slot, block)
+// One CUDA graph holds graph_k iterations of [axpy, step, sweeps] for each equation kind present, a
+// branch per kind and sort of slot; every launch covers all slots of that kind through a work list of (slot, block)
 // pairs, so instances of different sizes share one launch.  A host worker thread admits queued
 // requests when a slot and arena space are free, relaunches the graph, and retires finished
 // slots while the others keep running (continuous batching).
@@ -998,7 +999,14 @@ void worker_loop(rd_batch* b) {
         changed = true;
       }
     }
-    if (changed && rebuild_items(b) != RD_OK) b->worker_error = rd_last_error();
+    // without its work lists a graph must not run: they may name slots that changed since, or be freed
+    if (changed && rebuild_items(b) != RD_OK) {
+      b->worker_error = rd_last_error();
+      std::lock_guard<std::mutex> lk(b->mu);
+      b->stop = true;
+      b->cv.notify_all();
+      return;
+    }
     int active = 0;
     for (const SlotHost& sh : b->slots) active += sh.used;
     if (active == 0) {
@@ -1041,7 +1049,13 @@ void worker_loop(rd_batch* b) {
     // graph, whose capture takes as long as several sweeps, stay until half their slots are gone (or
     // a request is admitted)
     b->stale += retired;
-    if (retired && running > 0 && b->stale >= running) rebuild_items(b);
+    if (retired && running > 0 && b->stale >= running && rebuild_items(b) != RD_OK) {
+      b->worker_error = rd_last_error();
+      std::lock_guard<std::mutex> lk(b->mu);
+      b->stop = true;
+      b->cv.notify_all();
+      return;
+    }
   }
 }
 
