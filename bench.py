@@ -654,7 +654,7 @@ def main():
                          "(for profilers, which cannot attribute kernels inside conditional nodes)")
     ap.add_argument("--upd-rows", type=int, default=0, help="rows per CTA of k_upd (0: as --band-rows)")
     ap.add_argument("--fused-update", type=int, default=1, choices=(0, 1),
-                    help="1: the update of each PDHG iteration fused with the next residual (k_updres)")
+                    help="1: the primal update of each PDHG iteration fused with the next residual (k_primal)")
     ap.add_argument("--dc-stall-window", type=int, default=None,
                     help="defect correction: stop the FP32 inner solve when its residual has not halved "
                          "for this many updates (default: the library's)")

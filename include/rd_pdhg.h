@@ -184,8 +184,9 @@ typedef struct {
                              time; 0: one looped pass body for every pass                       */
     int autotune;         /* 1: at create, time each sweep kernel over a few PDHG iterations at
                              every tile that fits and keep the fastest per kernel (band rows of
-                             k_res and of the update, column width of the column solve; ignored when band_rows
-                             or col_width is set); 0 (default): the occupancy-based planner.
+                             k_res and of the update, column width of the column solve; ignored
+                             when band_rows or col_width is set); 0 (default): the occupancy-based
+                             planner.
                              Timing noise can change the choice between runs, and with it the
                              summation order of the stopping norm (results agree to rounding). */
     int dc_stall_window;  /* DC: the FP32 inner solve also stops (as converged) when its residual
@@ -370,8 +371,9 @@ typedef struct {
 
 /* Create a batch: arena of hbm_budget_bytes (allocated here, once), at most max_slots requests
  * resident at a time, solver options (graph_k, max_iter, dc_inner_rtol, dc_max_outer, omega,
- * small_solve, autotune; NULL = defaults), work issued on cuda_stream.  (autotune has no
- * effect: the launch shapes of the batched kernels follow from the grids.)  Starts the library's scheduling thread. */
+ * small_solve; NULL = defaults), work issued on cuda_stream.  Starts the library's scheduling
+ * thread.  (autotune has no effect here: the launch shapes of the batched kernels follow from the
+ * grids.) */
 RD_API rd_status rd_batch_create(rd_batch **out, size_t hbm_budget_bytes, int max_slots,
                                  const rd_opts *opts, void *cuda_stream);
 

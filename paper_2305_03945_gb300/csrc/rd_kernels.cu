@@ -1,9 +1,13 @@
 // Step-level sm_103a kernels of the PDHG solver (arxiv 2305.03945, Section 2.1, Algorithm 1):
 // the step set-up, the FP64 residual of defect correction, the FP64 update and the mass sum.
-// The per-iteration sweeps live in rd_sweep.cuh (instantiated per equation group in rd_sweep_{f32,f64}_{lap,bih}.cu,
-// rd_fused_{lap,bih}.cu and rd_sweep_col.cu).
+// The per-iteration sweeps live in rd_band.cuh (register-resident transforms, the default on 2-D
+// grids with sides of 16 points and more; instantiated in rd_band_lines.cu and
+// rd_band_{f32,f64}_{lap,two,bih}.cu) and in rd_sweep.cuh (shared-memory transforms, for the grids
+// and options the former do not take; instantiated in rd_sweep_{f32,f64}_{lap,bih}.cu and
+// rd_sweep_col.cu).
 //
-// One PDHG iteration is three launches:
+// One PDHG iteration of rd_sweep.cuh is three launches (rd_band.cuh regroups the same work as
+// k_fcol, k_dual and k_primal):
 //   k_res  (row bands)      W = F(U_n) (eq. F(U) rd equation / F(U) CH / Section 3.4.1), the
 //                           per-band partial sums of ||W_c||^2, the forward row transform of W
 //                           along x, and (last block of the instance) the stopping decision

@@ -1,4 +1,6 @@
-// The three kernels of one G-prox PDHG iteration (arxiv 2305.03945, Section 2.1, Algorithm 1),
+// The three kernels of one G-prox PDHG iteration (arxiv 2305.03945, Section 2.1, Algorithm 1) on
+// shared-memory transforms: the form of sides below 16 points, of rd_opts.fused_update = 0, and the
+// stencils, reactions and descriptors that rd_band.cuh, rd_cube.cuh and rd_3d.cuh build on.  Kernels
 // templated on the arithmetic type T and on the equation K so that each instantiation holds only
 // its own physics.  T = float is the inner solve of FP64 defect correction (the unknown is the
 // correction d of u + d); T = double is the plain FP64 method.
