@@ -166,8 +166,8 @@ __device__ __forceinline__ void fcol_body(const Desc& d, int blk, unsigned char*
 // and takes up to 255 (the same rule as band_threads_max).
 template <class T, int V>
 struct BandThreads { static constexpr int value = sizeof(T) == 8 && V == 16 ? 256 : 512; };
-// of k_fcol: FP32 lines of 4096 and 8192 points take 1024 threads (at 64 registers, without spills
-// once the boundary kind is fixed at compile time) to hold two lines or more
+// of k_fcol: FP32 lines of 4096 and 8192 points take 1024 threads to hold two lines or more; at 64
+// registers these and the 2048-point ones spill 150 to 210 bytes (k_fcol_tma 50 to 110)
 template <class T, int LOGN, int V>
 struct ColThreads {
   static constexpr int value = LOGN >= 12 && sizeof(T) == 4 ? 1024 : BandThreads<T, V>::value;
