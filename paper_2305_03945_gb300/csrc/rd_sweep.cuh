@@ -341,12 +341,6 @@ __device__ __forceinline__ void vst(T* __restrict__ p, const T* v) {
   }
 }
 
-// two adjacent entries of an array as one 8- or 16-byte load
-template <class T>
-__device__ __forceinline__ cx<T> ld_pair(const T* p) {
-  return *reinterpret_cast<const cx<T>*>(p);
-}
-
 // Copy rows g0 .. g0+nrows-1 (boundary-mapped) of a plane into shared memory (row stride nx).
 // Each thread first gathers up to 8 vectors into registers and only then stores them, so that
 // all of its global loads are in flight together.
