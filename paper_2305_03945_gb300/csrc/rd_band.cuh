@@ -554,13 +554,19 @@ struct Pt4 {
 template <int K>
 __host__ __device__ constexpr int ncomp_of() { return KT<K>::two ? 2 : 1; }
 
-// Shared-memory bytes of a k_primal block: the band's rows of U with H halo rows, then reused by
-// the line buffers of the forward transform; and in front the table of row offsets.
+// Bytes of a k_primal block's table of row offsets, (rows + 2H)(2H + 1) of them: whole 16-byte vectors, since
+// what lies behind it is read and written in such.
+__host__ __device__ constexpr int primal_table_bytes(int rows, int H) {
+  return ((rows + 2 * H) * (2 * H + 1) * (int)sizeof(int) + 15) / 16 * 16;
+}
+
+// Shared-memory bytes of a k_primal block: the table, and behind it the band's rows of U with H halo rows,
+// whose place the line buffers of the forward transform take afterwards.
 template <class T>
 __host__ __device__ inline int primal_smem_bytes(int nc, int rows, int H, int nx, int line_len, int line_bufs) {
   const int u = nc * (rows + 2 * H) * nx * (int)sizeof(T);
   const int l = line_bufs * line_len * (int)sizeof(cx<T>);
-  return (u > l ? u : l) + (rows + 2 * H) * (2 * H + 1) * (int)sizeof(int);
+  return primal_table_bytes(rows, H) + (u > l ? u : l);
 }
 
 // Threads of a k_primal block at most, and the blocks an SM shall hold (the register cap).  FP32 lines of
@@ -596,8 +602,7 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
   // updated exactly as the row it maps to, by that row's neighbours); mapped per group of four points they
   // cost 7% of the kernel's instructions (steps: 1024 x 128 805 -> 782 us, 512^2 716 -> 705 us)
   int* roff = reinterpret_cast<int*>(smem_raw);
-  const int tab = (srows * (2 * H + 1) + 3) / 4 * 4;
-  T* us = reinterpret_cast<T*>(smem_raw + tab * sizeof(int));
+  T* us = reinterpret_cast<T*>(smem_raw + primal_table_bytes(rows, H));
   for (int k = tid; k < srows * (2 * H + 1); k += nt) {
     const int r = k / (2 * H + 1), di = k - r * (2 * H + 1) - H;
     roff[k] = bcmap(bcmap(y0 + r - H, ny, bc) + di, ny, bc) << LOGN;
