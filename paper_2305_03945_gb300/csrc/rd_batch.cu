@@ -346,6 +346,12 @@ struct SlotHost {
   bool fast = false; // every side 16 points or more: the line kernels of rd_batch_lines.cuh
   int small = 0;     // a 2-D request whose inner solves run in one launch (1 one block, 2 a cluster)
   Desc d32{}, d64{};
+  // what else admission copies to the device.  A copy from pageable memory may read its source after the
+  // call has returned (it does where the device reads host memory through the host's page tables), so the
+  // sources live here until the stream has been synchronised: no wait per admission.
+  std::vector<double> u0;
+  std::vector<float> mu;
+  Slot ctl{};
 };
 
 size_t slot_bytes(const rd_request& r, size_t* npts_out) {
@@ -411,6 +417,7 @@ struct rd_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   bool graph_dirty = true;
+  bool lists_dirty = false;  // the slots have changed since the work lists were built
   int smem_sweep = 0;
   int smem_sweep2 = 0;  // the band kernels of the two-species kinds
   // queues.  mu guards the queues, outputs, stats, worker_error, stop and the arena's free list
@@ -599,7 +606,8 @@ rd_status rebuild_graph(rd_batch* b) {
   return RD_OK;
 }
 
-// Upload the work lists of all groups from the slot table.
+// Upload the work lists of all groups from the slot table; at most once between two synchronisations of the
+// stream (the copies may still read the host lists of the last time until then).
 rd_status rebuild_items(rd_batch* b) {
   for (int g = 0; g < kBatchGroups; ++g) {
     rd_batch::Lists& l = b->lists[g];
@@ -650,6 +658,7 @@ rd_status rebuild_items(rd_batch* b) {
     }
   }
   b->graph_dirty = true;
+  b->lists_dirty = false;
   b->stale = 0;
   return RD_OK;
 }
@@ -748,11 +757,11 @@ void admit3(rd_batch* b, Request& q, int s, char* mem, size_t npts, rd_status* e
   sh.d32 = d32;
   sh.d64 = d64;
   sh.nd3 = true;
-  std::vector<float> all_mu;
   const int n_ax[3] = {nx, ny, nz};
   const double h_ax[3] = {hx, hy, hz};
-  for (int a = 0; a < 3; ++a) append_mu(b, n_ax[a], r.bc == RD_BC_NEUMANN, h_ax[a], all_mu);
-  Slot ctl{};
+  for (int a = 0; a < 3; ++a) append_mu(b, n_ax[a], r.bc == RD_BC_NEUMANN, h_ax[a], sh.mu);
+  sh.u0 = std::move(q.u0);
+  Slot& ctl = sh.ctl;
   ctl.outer.max_iter = 1 << 30;
   ctl.inner.max_iter = b->opts.max_iter;
   ctl.phase = PH_BEGIN;
@@ -763,12 +772,11 @@ void admit3(rd_batch* b, Request& q, int s, char* mem, size_t npts, rd_status* e
   ctl.tol_kind = r.tol_kind;
   cudaStream_t st = b->stream;
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(mus, all_mu.data(), all_mu.size() * 4, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(u, q.u0.data(), npts * 8, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mus, sh.mu.data(), sh.mu.size() * 4, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(u, sh.u0.data(), npts * 8, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d32 + s, &sh.d32, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d64 + s, &sh.d64, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_slots + s, &ctl, sizeof(Slot), cudaMemcpyHostToDevice, st);
-  // (no wait: the copies read pageable memory, which cudaMemcpyAsync has staged when it returns)
   if (e != cudaSuccess) *err = bfail(RD_ERR_CUDA, std::string("admission: ") + cudaGetErrorString(e));
 }
 
@@ -898,10 +906,10 @@ bool admit(rd_batch* b, Request& q, rd_status* err) {
   sh.d32 = d32;
   sh.d64 = d64;
   // eigenvalues, state, control block
-  std::vector<float> all_mu;
-  append_mu(b, nx, r.bc == RD_BC_NEUMANN, hx, all_mu);
-  append_mu(b, ny, r.bc == RD_BC_NEUMANN, hy, all_mu);
-  Slot ctl{};
+  append_mu(b, nx, r.bc == RD_BC_NEUMANN, hx, sh.mu);
+  append_mu(b, ny, r.bc == RD_BC_NEUMANN, hy, sh.mu);
+  sh.u0 = std::move(q.u0);
+  Slot& ctl = sh.ctl;
   ctl.outer.max_iter = 1 << 30;
   ctl.inner.max_iter = b->opts.max_iter;
   ctl.phase = PH_BEGIN;
@@ -912,12 +920,11 @@ bool admit(rd_batch* b, Request& q, rd_status* err) {
   ctl.tol_kind = r.tol_kind;
   cudaStream_t st = b->stream;
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(mus, all_mu.data(), all_mu.size() * 4, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(u, q.u0.data(), npts * 8, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mus, sh.mu.data(), sh.mu.size() * 4, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(u, sh.u0.data(), npts * 8, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d32 + s, &sh.d32, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_d64 + s, &sh.d64, sizeof(Desc), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_slots + s, &ctl, sizeof(Slot), cudaMemcpyHostToDevice, st);
-  // (no wait: the copies read pageable memory, which cudaMemcpyAsync has staged when it returns)
   if (e != cudaSuccess) *err = bfail(RD_ERR_CUDA, std::string("admission: ") + cudaGetErrorString(e));
   std::lock_guard<std::mutex> lk(b->mu);
   b->stats.admitted += 1;
@@ -961,8 +968,8 @@ void retire(rd_batch* b, int s, const Slot& ctl) {
   res.t_done = now_s();
   char* mem = sh.mem;
   const size_t mem_bytes = sh.mem_bytes;
-  Slot idle{};
-  cudaMemcpyAsync(b->d_slots + s, &idle, sizeof(Slot), cudaMemcpyHostToDevice, b->stream);
+  static_assert(PH_IDLE == 0, "a cleared control block is an idle slot's");
+  cudaMemsetAsync(b->d_slots + s, 0, sizeof(Slot), b->stream);
   sh = SlotHost{};
   std::lock_guard<std::mutex> lk(b->mu);
   b->arena.release(mem, mem_bytes);
@@ -976,7 +983,6 @@ void worker_loop(rd_batch* b) {
   cudaStream_t st = b->stream;
   while (true) {
     // admit what fits
-    bool changed = false;
     {
       std::unique_lock<std::mutex> lk(b->mu);
       int active = 0;
@@ -996,16 +1002,8 @@ void worker_loop(rd_batch* b) {
           break;
         }
         if (err != RD_OK) b->worker_error = rd_last_error();
-        changed = true;
+        b->lists_dirty = true;
       }
-    }
-    // without its work lists a graph must not run: they may name slots that changed since, or be freed
-    if (changed && rebuild_items(b) != RD_OK) {
-      b->worker_error = rd_last_error();
-      std::lock_guard<std::mutex> lk(b->mu);
-      b->stop = true;
-      b->cv.notify_all();
-      return;
     }
     int active = 0;
     for (const SlotHost& sh : b->slots) active += sh.used;
@@ -1014,7 +1012,8 @@ void worker_loop(rd_batch* b) {
       if (b->stop && b->queue.empty()) return;
       continue;
     }
-    if (b->graph_dirty && rebuild_graph(b) != RD_OK) {
+    // without its work lists a graph must not run: they may name slots that changed since, or be freed
+    if ((b->lists_dirty && rebuild_items(b) != RD_OK) || (b->graph_dirty && rebuild_graph(b) != RD_OK)) {
       b->worker_error = rd_last_error();
       std::lock_guard<std::mutex> lk(b->mu);
       b->stop = true;
@@ -1037,6 +1036,8 @@ void worker_loop(rd_batch* b) {
     int retired = 0, running = 0;
     for (int s = 0; s < b->max_slots; ++s) {
       if (!b->slots[s].used) continue;
+      std::vector<double>().swap(b->slots[s].u0);  // the admission's copies have run
+      std::vector<float>().swap(b->slots[s].mu);
       const Slot ctl = b->h_slots[s];
       if (ctl.phase == PH_DONE || ctl.phase == PH_FAILED) {
         retire(b, s, ctl);
@@ -1049,13 +1050,7 @@ void worker_loop(rd_batch* b) {
     // graph, whose capture takes as long as several sweeps, stay until half their slots are gone (or
     // a request is admitted)
     b->stale += retired;
-    if (retired && running > 0 && b->stale >= running && rebuild_items(b) != RD_OK) {
-      b->worker_error = rd_last_error();
-      std::lock_guard<std::mutex> lk(b->mu);
-      b->stop = true;
-      b->cv.notify_all();
-      return;
-    }
+    if (retired && running > 0 && b->stale >= running) b->lists_dirty = true;
   }
 }
 
@@ -1217,7 +1212,7 @@ void rd_batch_destroy(rd_batch* b) {
     }
     b->worker.join();
   }
-  if (b->stream) cudaStreamSynchronize(b->stream);
+  cudaStreamSynchronize(b->stream);  // (NULL: the legacy default stream, whose copies read the slots' memory too)
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->graph) cudaGraphDestroy(b->graph);
   for (rd_batch::Lists& l : b->lists)

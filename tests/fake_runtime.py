@@ -48,12 +48,12 @@ def names(fn):
     return buf.value.decode().split("\n")[:-1]
 
 
-def run(path, script, timeout=300):
+def run(path, script, timeout=300, env=None):
     """Runs ``script`` in a child process whose ``rd`` and ``lib`` are this build's; returns its output."""
     head = ("import sys; sys.path.insert(0, %r); sys.path.insert(0, %r)\n"
             "import fake_runtime as F\nrd, lib = F.load(%r)\n" % (ROOT, os.path.join(ROOT, "tests"), path))
     r = subprocess.run([sys.executable, "-c", head + script], stdout=subprocess.PIPE, stderr=subprocess.STDOUT,
-                       timeout=timeout, cwd=ROOT)
+                       timeout=timeout, cwd=ROOT, env={**os.environ, **(env or {})})
     out = r.stdout.decode(errors="replace")
     assert r.returncode == 0, out
     return out

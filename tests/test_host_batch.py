@@ -1,0 +1,52 @@
+"""The batch server's host side (CPU), on a CUDA runtime in which an asynchronous copy runs as late as it may:
+at the next synchronisation, reading its source then.  A graph launch finishes every step it finds begun, so
+a request's result is its initial state, as far as the copies in and out are sound."""
+import shutil
+
+import pytest
+
+import fake_runtime as F
+
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+
+SERVE = """
+import time
+import numpy as np
+from paper_2305_03945_gb300 import workloads as WL
+
+def request(k, shape):
+    nz, ny, nx = (1,) * (3 - len(shape)) + shape
+    pb = WL.Problem(nx=nx, ny=ny, nz=nz, lx=1.0, ly=1.0, lz=1.0, bc="neumann" if k % 2 else "periodic", op="laplacian",
+                    kind="allen_cahn", dt=1e-3, a=0.05, b=20.0, tol=1e-11, tol_kind="f_rel")
+    return pb, WL.rng(k).standard_normal(pb.shape)
+
+def drain(b, ids, t_max=30.0):
+    got, t0 = {}, time.time()
+    while len(got) < len(ids) and time.time() - t0 < t_max:
+        for r in b.poll(timeout=0.2):
+            got[r["id"]] = r
+    return got
+
+def serve(b, reqs):
+    ids = [b.submit(pb, u0, 1, tag=k) for k, (pb, u0) in enumerate(reqs)]
+    got = drain(b, ids)
+    assert len(got) == len(ids), "requests that never finished"
+    for (rid, out), (pb, u0) in zip(ids, reqs):
+        assert got[rid]["status"] == 0, got[rid]
+        assert np.array_equal(out, u0), pb.shape
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return F.build(str(tmp_path_factory.mktemp("fake") / "fake.so"))
+
+
+def test_admission_keeps_its_sources_until_the_copies_have_run(lib):
+    """More requests than slots (slots are used again), 2-D and 3-D, sizes on the heap and mapped."""
+    F.run(lib, SERVE + """
+lib.fake_slots(3)
+shapes = [(64, 64), (8, 16, 16), (16, 16), (256, 512), (128, 32), (32, 32, 32), (4, 8), (512, 64)]
+with rd.Batch(1 << 26, 3, stream=0) as b:
+    serve(b, [request(k, s) for k, s in enumerate(shapes)])
+""", env={"MALLOC_PERTURB_": "165"})
