@@ -252,6 +252,10 @@ constexpr int kBatchBandRows = 4;
 constexpr int kBatchColWidth = 4;
 constexpr int kBatchGroups = 7;         // equation kinds served
 constexpr int kBatchParts = 5;          // branches of a group's graph: see launch_branch
+// Entries one slot adds to the work lists at most.  2-D: ny / 4 bands, and ny / 2 blocks of the line kernels or
+// 2 nx / 4 column blocks of two components; 3-D: its blocks.
+constexpr int kBatchSlotItems =
+    std::max(kBatchMaxSide / kBatchBandRows + std::max(kBatchMaxSide / 2, 2 * kBatchMaxSide / kBatchColWidth), kBatchMaxBlk3);
 const int kGroupKey[kBatchGroups] = {KK_NONE_LAP, KK_AC, KK_CH_IMPL, KK_CH_SPLIT, KK_NONE_BIH, KK_GS, KK_SCHNAK};
 
 double now_s() {
@@ -304,26 +308,11 @@ struct Arena {
   }
 };
 
-// A work list of (slot, block) pairs: built on the host, copied to a device array that grows to fit.
+// A work list of (slot, block) pairs: built on the host, and its part of the batch's device array (rd_batch::d_items).
 struct ItemList {
   int2* d = nullptr;
-  int cap = 0, n = 0;
+  int n = 0;
   std::vector<int2> h;
-  cudaError_t upload(cudaStream_t s) {
-    n = (int)h.size();
-    if (n == 0) return cudaSuccess;
-    if (n > cap) {
-      if (d) cudaFree(d);
-      d = nullptr;
-      cap = std::max(2 * n, 1024);
-      const cudaError_t e = cudaMalloc(&d, sizeof(int2) * cap);
-      if (e != cudaSuccess) {
-        cap = 0;
-        return e;
-      }
-    }
-    return cudaMemcpyAsync(d, h.data(), n * sizeof(int2), cudaMemcpyHostToDevice, s);
-  }
 };
 
 struct Request {
@@ -402,6 +391,8 @@ struct rd_batch {
     int smem_line2[2] = {}, smem_line3[2] = {};  // row and column kernels
     int thr3[3] = {}, smem3[3] = {};             // transform passes of the old3 slots
   } lists[kBatchGroups];
+  int2* d_items = nullptr;   // the entries of all lists, kBatchSlotItems per slot (allocated once: serving
+  int2* h_items = nullptr;   // allocates no device memory but the graph's), and their pinned source
   int smem_usable = 0;
   // one capture stream and join event per branch of the graph (see rebuild_graph)
   cudaStream_t branch_stream[kBatchParts * kBatchGroups] = {};
@@ -606,8 +597,8 @@ rd_status rebuild_graph(rd_batch* b) {
   return RD_OK;
 }
 
-// Upload the work lists of all groups from the slot table; at most once between two synchronisations of the
-// stream (the copies may still read the host lists of the last time until then).
+// Upload the work lists of all groups from the slot table, one behind the other; at most once between two
+// synchronisations of the stream (the copy may still read the entries of the last time until then).
 rd_status rebuild_items(rd_batch* b) {
   for (int g = 0; g < kBatchGroups; ++g) {
     rd_batch::Lists& l = b->lists[g];
@@ -650,13 +641,20 @@ rd_status rebuild_items(rd_batch* b) {
       list(l.col, d.ncomp * d.ncolblk);
     }
   }
+  size_t n = 0;
+  const size_t cap = (size_t)b->max_slots * kBatchSlotItems;
   for (int g = 0; g < kBatchGroups; ++g) {
     rd_batch::Lists& l = b->lists[g];
     for (ItemList* it : {&l.band, &l.col, &l.small_phase, &l.small1, &l.small2, &l.line_phase, &l.line2, &l.old3, &l.line3}) {
-      const cudaError_t e = it->upload(b->stream);
-      if (e != cudaSuccess) return bfail(RD_ERR_CUDA, cudaGetErrorString(e));
+      if (n + it->h.size() > cap) return bfail(RD_ERR_CUDA, "batch work lists beyond their bound");
+      it->d = b->d_items + n;
+      it->n = (int)it->h.size();
+      std::copy(it->h.begin(), it->h.end(), b->h_items + n);
+      n += it->h.size();
     }
   }
+  const cudaError_t e = cudaMemcpyAsync(b->d_items, b->h_items, n * sizeof(int2), cudaMemcpyHostToDevice, b->stream);
+  if (e != cudaSuccess) return bfail(RD_ERR_CUDA, cudaGetErrorString(e));
   b->graph_dirty = true;
   b->lists_dirty = false;
   b->stale = 0;
@@ -1088,6 +1086,8 @@ rd_status rd_batch_create(rd_batch** out, size_t hbm_budget_bytes, int max_slots
   if ((e = cudaMalloc(&b->d_d32, sizeof(Desc) * max_slots)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_d64, sizeof(Desc) * max_slots)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_slots, sizeof(Slot) * max_slots)) != cudaSuccess ||
+      (e = cudaMalloc(&b->d_items, sizeof(int2) * max_slots * kBatchSlotItems)) != cudaSuccess ||
+      (e = cudaMallocHost(&b->h_items, sizeof(int2) * max_slots * kBatchSlotItems)) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_slots, sizeof(Slot) * max_slots)) != cudaSuccess)
     return cleanup(bfail(RD_ERR_OOM, cudaGetErrorString(e)));
   cudaMemset(b->d_slots, 0, sizeof(Slot) * max_slots);
@@ -1215,9 +1215,8 @@ void rd_batch_destroy(rd_batch* b) {
   cudaStreamSynchronize(b->stream);  // (NULL: the legacy default stream, whose copies read the slots' memory too)
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->graph) cudaGraphDestroy(b->graph);
-  for (rd_batch::Lists& l : b->lists)
-    for (ItemList* it : {&l.band, &l.col, &l.small_phase, &l.small1, &l.small2, &l.line_phase, &l.line2, &l.old3, &l.line3})
-      if (it->d) cudaFree(it->d);
+  if (b->d_items) cudaFree(b->d_items);
+  if (b->h_items) cudaFreeHost(b->h_items);
   if (b->d_tables) cudaFree(b->d_tables);
   if (b->d_d32) cudaFree(b->d_d32);
   if (b->d_d64) cudaFree(b->d_d64);

@@ -50,3 +50,19 @@ shapes = [(64, 64), (8, 16, 16), (16, 16), (256, 512), (128, 32), (32, 32, 32), 
 with rd.Batch(1 << 26, 3, stream=0) as b:
     serve(b, [request(k, s) for k, s in enumerate(shapes)])
 """, env={"MALLOC_PERTURB_": "165"})
+
+
+def test_serving_allocates_no_device_memory(lib):
+    """With device memory exhausted once the batch is made, requests of every route are still served."""
+    F.run(lib, SERVE + """
+lib.fake_slots(4)
+with rd.Batch(1 << 28, 4, stream=0) as b:
+    serve(b, [request(0, (64, 64))])
+    lib.fake_refuse_alloc(1)
+    n = lib.fake_alloc_calls()
+    shapes = [(1024, 1024), (512, 1024), (1024, 4), (4, 1024), (128, 128), (16, 16), (4, 4), (64, 64, 64), (4, 32, 32), (16, 512, 16)]
+    serve(b, [request(k, s) for k, s in enumerate(shapes)])
+    serve(b, [request(k, (1024, 1024)) for k in range(8)])
+    assert lib.fake_alloc_calls() == n
+    lib.fake_refuse_alloc(0)
+""")
