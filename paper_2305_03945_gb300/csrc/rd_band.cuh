@@ -670,7 +670,6 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
   constexpr int MI = V / 4 / NC > 0 ? V / 4 / NC : 1;  // groups per thread at most (a thread per V values of a line)
   const int groups = (rows >> 1) << LV;
   T w[MI][NC][2][4];
-  T acc[2] = {T(0), T(0)};
 #pragma unroll
   for (int m = 0; m < MI; ++m) {
     const int g = tid + m * nt;
@@ -697,10 +696,7 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
             T ww[2] = {T(0), T(0)};
             residual_pt<T, K, DC>(d, x[0], x[NC - 1], b0, b1, 0, q, rr[0][q], NC == 2 ? rr[1][q] : T(0), ww);
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-              w[m][c][h][q] = ww[c];
-              acc[c] += ww[c] * ww[c];
-            }
+            for (int c = 0; c < NC; ++c) w[m][c][h][q] = ww[c];
           }
         };
         if constexpr (BASE && HB > 0) {
@@ -725,13 +721,18 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
   cx<T>* lines = reinterpret_cast<cx<T>*>(us);
   constexpr int LEN = Lay<T, LOGN, V, false>::len;
   const int hr = rows >> 1;
+  SumSq<T> acc[NC];  // (summed here, not beside the stencils that need the registers)
 #pragma unroll
   for (int m = 0; m < MI; ++m) {
     const int g = tid + m * nt;
     if (g < groups) {
       const int pr = g >> LV, j0 = (g & ((1 << LV) - 1)) * 4;
 #pragma unroll
-      for (int c = 0; c < NC; ++c) put4(lines + (c * hr + pr) * LEN, N, per, j0, w[m][c][0], w[m][c][1]);
+      for (int c = 0; c < NC; ++c) {
+        put4(lines + (c * hr + pr) * LEN, N, per, j0, w[m][c][0], w[m][c][1]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[c].add(w[m][c][q >> 2][q & 3]);
+      }
     }
   }
   __syncthreads();
@@ -749,8 +750,8 @@ __device__ __forceinline__ void primal_body(const Desc& d, State* __restrict__ s
   }
 
   // 4. partial norms, ticket, stopping decision in the last block
-  const double s0 = block_sum((double)acc[0], red);
-  const double s1 = NC == 2 ? block_sum((double)acc[1], red) : 0.0;
+  const double s0 = block_sum(acc[0].value(), red);
+  const double s1 = NC == 2 ? block_sum(acc[NC - 1].value(), red) : 0.0;
   if (tid == 0) {
     d.partials[band] = s0;
     if (NC == 2) d.partials[d.nupd + band] = s1;

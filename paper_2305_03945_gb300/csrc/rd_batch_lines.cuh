@@ -95,7 +95,7 @@ __device__ __forceinline__ bool slot_inner(const Slot* sl) { return *((volatile 
 
 // W = F(U_n) on the row pairs of group `grp` and its forward row transform into WY
 template <int K, int LOGN, int V>
-__device__ __forceinline__ void rowres2_body(const Desc& d, int grp, unsigned char* smem_raw, float* acc_out) {
+__device__ __forceinline__ void rowres2_body(const Desc& d, int grp, unsigned char* smem_raw, double* acc_out) {
   using F = Rf<LOGN, V>;
   constexpr int N = F::N;
   constexpr int H = KT<K>::H;
@@ -113,7 +113,7 @@ __device__ __forceinline__ void rowres2_body(const Desc& d, int grp, unsigned ch
   const float* X = static_cast<const float*>(d.X);
   const float* Bs = static_cast<const float*>(d.base);
   const float* R = static_cast<const float*>(d.rhs);
-  float acc[2] = {0.f, 0.f};
+  SumSq<float> acc[NC];
 #pragma unroll 1
   for (int m = 0; m < V / 4; ++m) {
     const int j0 = 4 * (t + m * F::TPL);
@@ -140,7 +140,7 @@ __device__ __forceinline__ void rowres2_body(const Desc& d, int grp, unsigned ch
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
             w[c][h][q] = ww[c];
-            acc[c] += ww[c] * ww[c];
+            acc[c].add(ww[c]);
           }
         }
       };
@@ -170,8 +170,8 @@ __device__ __forceinline__ void rowres2_body(const Desc& d, int grp, unsigned ch
     row_forward<float, LOGN, V>(d, lines + (c * lpb + lline) * LEN, static_cast<float*>(d.WY) + c * plane + (size_t)row0 * N, t,
                                 live, sync);
   if (live) {
-    acc_out[0] += acc[0];
-    acc_out[1] += acc[1];
+    acc_out[0] += acc[0].value();
+    if constexpr (NC == 2) acc_out[1] += acc[1].value();
   }
 }
 
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kLineThreads)
   load_desc(sd, descs + w.x);
   __syncthreads();
   const Desc& d = sd;
-  float acc[2] = {0.f, 0.f};
+  double acc[2] = {0.0, 0.0};
   batch_len<D3>(d.lognx, [&](auto l, auto v) {
     constexpr int L = decltype(l)::value, V = decltype(v)::value;
     const int lpb = kLineThreads / Rf<L, V>::TPL;

@@ -66,9 +66,10 @@ struct Pt4z {
 // ---------------------------------------------------------------------------------------
 // k3_rowres
 // ---------------------------------------------------------------------------------------
-// The lines of group `blk`; the squares of the thread's residuals are added to acc_out.
+// The lines of group `blk`; the squares of the thread's residuals are added to acc_out (in twice FP32's
+// precision, see SumSq).
 template <class T, int K, int LOGN, int V>
-__device__ __forceinline__ void rowres3_body(const Desc& d, int blk, unsigned char* smem_raw, T& acc_out) {
+__device__ __forceinline__ void rowres3_body(const Desc& d, int blk, unsigned char* smem_raw, double& acc_out) {
   using F = Rf<LOGN, V>;
   constexpr int N = F::N;
   constexpr int H = KT<K>::H;
@@ -85,7 +86,7 @@ __device__ __forceinline__ void rowres3_body(const Desc& d, int blk, unsigned ch
   const T* X = static_cast<const T*>(d.X);
   const T* Bs = static_cast<const T*>(d.base);
   const T* R = static_cast<const T*>(d.rhs);
-  T acc = T(0);
+  SumSq<T> acc;
 #pragma unroll 1
   for (int m = 0; m < V / 4; ++m) {
     const int j0 = 4 * (t + m * F::TPL);
@@ -100,7 +101,7 @@ __device__ __forceinline__ void rowres3_body(const Desc& d, int blk, unsigned ch
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           w[h][q] = residual3_pt<T, K, DC>(d, x, b, 0, 0, q, rr[q]);
-          acc += w[h][q] * w[h][q];
+          acc.add(w[h][q]);
         }
       };
       if constexpr (BASE && base_stencil<K>()) {
@@ -120,15 +121,15 @@ __device__ __forceinline__ void rowres3_body(const Desc& d, int blk, unsigned ch
   auto sync = [lline] { line_sync<F::TPL>(lline); };
   sync();
   row_forward<T, LOGN, V>(d, line, static_cast<T*>(d.WY) + o, t, live, sync);
-  if (live) acc_out += acc;
+  if (live) acc_out += acc.value();
 }
 
 // Partial norm of block `blk` of `nblk`, stopping decision in the last one.
-__device__ __forceinline__ void rowres_finish(const Desc& d, State* __restrict__ st, Slot* slot, int blk, int nblk, float a0,
-                                              float a1) {
+__device__ __forceinline__ void rowres_finish(const Desc& d, State* __restrict__ st, Slot* slot, int blk, int nblk, double a0,
+                                              double a1) {
   __shared__ double red[32];
-  const double s0 = block_sum((double)a0, red);
-  const double s1 = d.ncomp == 2 ? block_sum((double)a1, red) : 0.0;
+  const double s0 = block_sum(a0, red);
+  const double s1 = d.ncomp == 2 ? block_sum(a1, red) : 0.0;
   if (threadIdx.x == 0) {
     d.partials[blk] = s0;
     if (d.ncomp == 2) d.partials[nblk + blk] = s1;
@@ -141,9 +142,9 @@ __global__ void __launch_bounds__(256) k3_rowres(const __grid_constant__ Desc d,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
   if (!sweep_active(st, nullptr)) return;
-  T acc = T(0);
+  double acc = 0.0;
   rowres3_body<T, K, LOGN, V>(d, blockIdx.x, smem_raw, acc);
-  rowres_finish(d, st, nullptr, blockIdx.x, gridDim.x, acc, 0.f);
+  rowres_finish(d, st, nullptr, blockIdx.x, gridDim.x, acc, 0.0);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -570,6 +570,29 @@ __device__ __forceinline__ unsigned char* place_tables(unsigned char* smem, cons
   }
 }
 
+// A thread's share of a squared norm.  In FP32 the squares and their sum carry their rounding errors along
+// (Dot2 of Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26, 2005: the result is that of twice FP32's precision, to
+// n^2 2^-48 of it for n squares), ten FP32 operations per value; they are folded into an FP64 sum per line group.
+// Adding every square in FP64 instead costs a conversion and an addition on the FP64 pipes, two lanes per clock
+// and SM.  Step times with plain FP32 sums / these / FP64 sums: Gray-Scott 2048^2 x 2 8.09 / 8.14 / 9.49 ms, 8192^2
+// 42.5 / 43.8 / 50.1 ms, 128^3 1.918 / 1.919 / 2.00 ms, 1024^2 0.777 / 0.779 / 0.824 ms.
+template <class T>
+struct SumSq {
+  T s = T(0), c = T(0);
+  __device__ __forceinline__ void add(T w) {
+    if constexpr (sizeof(T) == 8) {
+      s += w * w;
+    } else {
+      const float p = __fmul_rn(w, w), e = __fmaf_rn(w, w, -p);
+      const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
+      const float d = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b));
+      s = t;
+      c = __fadd_rn(c, __fadd_rn(d, e));
+    }
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+
 // block-wide sum of a double, valid in thread 0; sh must hold 32 doubles
 __device__ __forceinline__ double block_sum(double v, double* sh) {
 #pragma unroll
