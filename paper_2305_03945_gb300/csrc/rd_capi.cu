@@ -825,9 +825,11 @@ rd_status autotune_plan(rd_pdhg* h, int H, int transform, int stage_base, int us
   // per-kernel time (ms, best of three) of kTuneIters iterations for one plan; false if it failed
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   for (int i = 0; i < 4; ++i) RD_CUDA(cudaEventCreate(&ev[i]));
-  auto iterate = [&](Desc& dt, const LaunchCfg& ct, cudaEvent_t* e, bool first) {
+  auto iterate = [&](Desc& dt, LaunchCfg ct, cudaEvent_t* e, bool first) {
     dt.fused = fused;
     dt.halo = halo.p;
+    CUtensorMap map;  // the column kernel the handle would run at this width
+    ct.tmap = h->dc && fused && make_col_map(dt, ct, &map) ? &map : nullptr;
     return fused ? launch_fused<T>(dt, dst, ct, s, e, first) : launch_iteration<T>(dt, dst, ct, s, e);
   };
   auto time_plan = [&](Desc& dt, const LaunchCfg& ct, float* kms) -> bool {
