@@ -244,19 +244,21 @@ __global__ void __launch_bounds__(TmaCol<LOGN>::threads, TmaCol<LOGN>::blocks)
   }
   __syncthreads();  // the barrier is initialised
   cx<float>* buf = reinterpret_cast<cx<float>*>(smem_tma) + m;
-  if (!mbar_wait0(mb)) {  // cannot happen while the memory system works; the tile stays as it was
-    if (threadIdx.x == 0) st->status = ST_DIVERGED;
-    mbar_wait0(mb);
-    return;
-  }
+  const bool here = mbar_wait0(mb);
   cx<float> v[V];
 #pragma unroll
   for (int e = 0; e < V; ++e) {
     const int n = P1::natural(t, e);
     v[e] = buf[(PER ? n : mk_perm(n, N)) * nl];
   }
+  // The wait cannot run out while the memory system works.  One thread's is the block's: all stop, the tile
+  // stays as it was and the solve ends with an error.
+  if (!__syncthreads_and(here)) {
+    if (threadIdx.x == 0) st->status = ST_FAULT;
+    mbar_wait0(mb);  // (the copies in flight write this block's shared memory)
+    return;
+  }
   auto sync = [] { __syncthreads(); };
-  sync();
   const cx<float>* tw = static_cast<const cx<float>*>(d.twy);
   rf_forward<float, LOGN, V, true>(v, buf, nl, tw, t, sync);
   const float* mux = static_cast<const float*>(d.mux);

@@ -397,6 +397,7 @@ rd_status status_of(int st) {
     case ST_CONVERGED: return RD_OK;
     case ST_NOT_CONVERGED: return RD_ERR_NOT_CONVERGED;
     case ST_DIVERGED: return RD_ERR_DIVERGED;
+    case ST_FAULT: return RD_ERR_CUDA;
     default: return RD_ERR_NOT_CONVERGED;
   }
 }
@@ -1398,7 +1399,9 @@ rd_status step_host(rd_pdhg* h, rd_step_info* info) {
   inf.status = status_of(final_status);
   if (info) *info = inf;
   if (inf.status != RD_OK)
-    return fail((rd_status)inf.status, inf.status == RD_ERR_DIVERGED ? "PDHG diverged" : "PDHG did not converge");
+    return fail((rd_status)inf.status, inf.status == RD_ERR_DIVERGED ? "PDHG diverged"
+                                       : inf.status == RD_ERR_CUDA   ? "a kernel's wait for its own copies ran out"
+                                                                     : "PDHG did not converge");
   return RD_OK;
 }
 
@@ -1430,7 +1433,9 @@ rd_status step_impl(rd_pdhg* h, rd_step_info* info) {
   inf.status = status_of(final_status);
   if (info) *info = inf;
   if (inf.status != RD_OK)
-    return fail((rd_status)inf.status, inf.status == RD_ERR_DIVERGED ? "PDHG diverged" : "PDHG did not converge");
+    return fail((rd_status)inf.status, inf.status == RD_ERR_DIVERGED ? "PDHG diverged"
+                                       : inf.status == RD_ERR_CUDA   ? "a kernel's wait for its own copies ran out"
+                                                                     : "PDHG did not converge");
   return RD_OK;
 }
 

@@ -12,7 +12,15 @@ enum Kind { RX_NONE = 0, RX_AC = 1, RX_CH_IMPL = 2, RX_CH_SPLIT = 3, RX_GS = 4, 
 enum Mode { MODE_PDHG = 0, MODE_PRECOND_ONLY = 1 };
 
 // per-solve status kept on the device
-enum StStatus { ST_ACTIVE = 0, ST_CONVERGED = 1, ST_NOT_CONVERGED = 2, ST_DIVERGED = 3, ST_IDLE = 4 };
+// (ST_FAULT: a bounded wait of a kernel ran out; the iterate says nothing)
+enum StStatus { ST_ACTIVE = 0, ST_CONVERGED = 1, ST_NOT_CONVERGED = 2, ST_DIVERGED = 3, ST_IDLE = 4, ST_FAULT = 5 };
+
+// Status of the outer loop of defect correction after an inner solve that ended with `inner`: active (the
+// correction is added) after convergence or the iteration limit.
+__host__ __device__ inline int outer_after_inner(int inner) {
+  if (inner == ST_CONVERGED || inner == ST_NOT_CONVERGED) return ST_ACTIVE;
+  return inner == ST_FAULT ? ST_FAULT : ST_DIVERGED;
+}
 
 constexpr double kDivergeFactor = 1e8;  // measure > 1e8 * first measure  ->  diverged
 constexpr int kRadix = 16;              // values each FFT thread holds per Stockham pass

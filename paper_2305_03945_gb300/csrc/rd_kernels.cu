@@ -180,11 +180,12 @@ __global__ void k_axpy_dc(double* __restrict__ u, const float* __restrict__ dlt,
   pdl_wait();
   if (*((volatile const int*)&outer->status) != ST_ACTIVE) return;
   const int is = *((volatile const int*)&inner->status);
-  const bool ok = is == ST_CONVERGED || is == ST_NOT_CONVERGED;
+  const int after = outer_after_inner(is);
+  const bool ok = after == ST_ACTIVE;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     outer->total += inner->n;
     outer->launches += (int)inner->trips;
-    if (!ok) outer->status = ST_DIVERGED;
+    if (!ok) outer->status = after;
   }
   if (!ok) return;
   const size_t n4 = n >> 2;
