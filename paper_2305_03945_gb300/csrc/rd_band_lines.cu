@@ -63,8 +63,9 @@ bool make_col_map(const Desc& d, const LaunchCfg& c, void* map) {
                                       CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <class T>
-cudaError_t launch_rowfwd(const Desc& d, const LaunchCfg& c, cudaStream_t s) {
+template <>
+cudaError_t launch_rowfwd<double>(const Desc& d, const LaunchCfg& c, cudaStream_t s) {
+  using T = double;
   return by_len<T>(d.lognx, c.vrow, [&](auto l, auto v) {
     constexpr int L = decltype(l)::value, V = decltype(v)::value;
     const int lpb = c.thr_dual / Rf<L, V>::TPL;
@@ -78,7 +79,9 @@ cudaError_t launch_dual(const Desc& d, State* st, const LaunchCfg& c, cudaStream
     constexpr int L = decltype(l)::value, V = decltype(v)::value;
     const int lpb = c.thr_dual / Rf<L, V>::TPL;
     const int grid = (d.ncomp * (d.ny / 2) + lpb - 1) / lpb;
-    return launch_pdl(pc ? k_dual<T, L, V, true> : k_dual<T, L, V, false>, grid, c.thr_dual, c.smem_dual, s, d, st);
+    if constexpr (sizeof(T) == 8)
+      if (pc) return launch_pdl(k_dual<T, L, V, true>, grid, c.thr_dual, c.smem_dual, s, d, st);
+    return pc ? cudaErrorNotSupported : launch_pdl(k_dual<T, L, V, false>, grid, c.thr_dual, c.smem_dual, s, d, st);
   });
 }
 
@@ -132,15 +135,17 @@ cudaError_t launch_fused(const Desc& d, State* st, const LaunchCfg& c, cudaStrea
 }
 
 template <class T>
-cudaError_t allow_band(const Desc& d, const LaunchCfg& c, int optin, bool primal) {
+cudaError_t allow_band(const Desc& d, const LaunchCfg& c, int optin, bool primal, bool tune) {
   cudaError_t e = cudaSuccess;
   if (c.transform && has_len<T>(d.logny, c.vcol))
     e = by_len<T>(d.logny, c.vcol, [&](auto l, auto v) {
       constexpr int L = decltype(l)::value, V = decltype(v)::value;
       if constexpr (sizeof(T) == 4 && V == 16 && L >= 11) {
-        const cudaError_t r =
-            d.bc == BC_PERIODIC ? allow_smem_k(k_fcol_tma<L, true>, optin) : allow_smem_k(k_fcol_tma<L, false>, optin);
-        if (r != cudaSuccess) return r;
+        if (c.tmap || tune) {
+          const cudaError_t r =
+              d.bc == BC_PERIODIC ? allow_smem_k(k_fcol_tma<L, true>, optin) : allow_smem_k(k_fcol_tma<L, false>, optin);
+          if (r != cudaSuccess || !tune) return r;
+        }
       }
       return d.bc == BC_PERIODIC ? allow_smem_k(k_fcol<T, L, V, true>, optin) : allow_smem_k(k_fcol<T, L, V, false>, optin);
     });
@@ -148,8 +153,11 @@ cudaError_t allow_band(const Desc& d, const LaunchCfg& c, int optin, bool primal
     e = by_len<T>(d.lognx, c.vrow, [&](auto l, auto v) {
       constexpr int L = decltype(l)::value, V = decltype(v)::value;
       cudaError_t r = allow_smem_k(k_dual<T, L, V, false>, optin);
-      if (r == cudaSuccess) r = allow_smem_k(k_dual<T, L, V, true>, optin);
-      return r != cudaSuccess ? r : allow_smem_k(k_rowfwd<T, L, V>, optin);
+      if constexpr (sizeof(T) == 8) {  // the preconditioner alone
+        if (r == cudaSuccess) r = allow_smem_k(k_dual<T, L, V, true>, optin);
+        if (r == cudaSuccess) r = allow_smem_k(k_rowfwd<T, L, V>, optin);
+      }
+      return r;
     });
   if (c.fast_row && primal && e == cudaSuccess) e = allow_primal<T>(d, c, optin);
   return e;
@@ -203,10 +211,9 @@ void plan_band(const Desc& d, int H, int smem_limit, LaunchCfg& c) {
 
 #define RD_BAND_COMMON(T)                                                                              \
   template cudaError_t launch_fcol<T>(const Desc&, State*, const LaunchCfg&, cudaStream_t, bool);      \
-  template cudaError_t launch_rowfwd<T>(const Desc&, const LaunchCfg&, cudaStream_t);                  \
   template cudaError_t launch_dual<T>(const Desc&, State*, const LaunchCfg&, cudaStream_t, bool);      \
   template cudaError_t launch_fused<T>(const Desc&, State*, const LaunchCfg&, cudaStream_t, cudaEvent_t*, bool); \
-  template cudaError_t allow_band<T>(const Desc&, const LaunchCfg&, int, bool);                        \
+  template cudaError_t allow_band<T>(const Desc&, const LaunchCfg&, int, bool, bool);                  \
   template void plan_band<T>(const Desc&, int, int, LaunchCfg&);
 RD_BAND_COMMON(float)
 RD_BAND_COMMON(double)

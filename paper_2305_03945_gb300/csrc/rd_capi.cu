@@ -1195,19 +1195,23 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
       RD_CUDA(launch_symbol(d, h->sym64, h->stream));
       h->h_desc[0].scale = h->h_desc[2].scale = h->sym64;
     }
-    RD_CUDA(h->dc ? allow_band<float>(d, c, optin, fused) : allow_band<double>(d, c, optin, fused));
+    const bool tune =
+        h->opts.autotune && !h->fch && !h->long2d && h->opts.band_rows == 0 && h->opts.col_width == 0 && h->opts.upd_rows == 0;
+    auto set_map = [&] { c.tmap = h->dc && fused && make_col_map(d, c, &h->colmap) ? &h->colmap : nullptr; };
+    set_map();
+    RD_CUDA(h->dc ? allow_band<float>(d, c, optin, fused, tune) : allow_band<double>(d, c, optin, fused, tune));
     if (!h->dc) h->cfgpc = c;
     const bool fch_new = h->fch && fch_fused(h->cfgpc);
     if (fch_new) RD_CUDA(allow_fch(d, h->cfgpc, optin));
     if (!fch_new && !(fused && c.fast_col))
       RD_CUDA(h->dc ? set_kernel_smem_limits<float>(nullptr) : set_kernel_smem_limits<double>(nullptr));
     share_tiles(h, d);
-    if (h->opts.autotune && !h->fch && !h->long2d && h->opts.band_rows == 0 && h->opts.col_width == 0 && h->opts.upd_rows == 0) {
+    if (tune) {
       const int stage_base = h->dc && (rx->kind == RD_RX_CH_IMPLICIT || rx->kind == RD_RX_CH_SPLIT);
       RD_TRY(h->dc ? autotune_plan<float>(h, H, transform, stage_base, usable, fused)
                    : autotune_plan<double>(h, H, transform, stage_base, usable, fused));
+      set_map();
     }
-    if (h->dc && fused && make_col_map(d, c, &h->colmap)) c.tmap = &h->colmap;
     if (fused) RD_TRY(h->dc ? plan_fused<float>(h, H) : plan_fused<double>(h, H));
     RD_CUDA(cudaMemcpy(h->d_desc, h->h_desc, 3 * sizeof(Desc), cudaMemcpyHostToDevice));
   }

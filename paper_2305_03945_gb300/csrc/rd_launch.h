@@ -44,7 +44,8 @@ template <class T>
 cudaError_t launch_col(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc);
 
 // The kernels of rd_band.cuh: launchers (rd_band_*.cu), the shared-memory limits of the ones the
-// plan (d, c) launches, and the planning rule of their launch shapes.
+// plan (d, c) launches (tune: and of those the tuner tries), and the planning rule of their launch shapes.  The
+// preconditioner alone (launch_rowfwd, pc = true) runs in double only.
 template <class T>
 cudaError_t launch_fcol(const Desc& d, State* st, const LaunchCfg& c, cudaStream_t s, bool pc);
 // Encodes the tensor map of d.WY for tiles of d.col_width columns into *map (a CUtensorMap) where
@@ -61,7 +62,7 @@ cudaError_t launch_primal_kind(const Desc& d, State* st, const LaunchCfg& c, cud
 template <class T, int K>
 cudaError_t allow_primal_kind(const Desc& d, const LaunchCfg& c, int optin);
 template <class T>
-cudaError_t allow_band(const Desc& d, const LaunchCfg& c, int optin, bool primal);
+cudaError_t allow_band(const Desc& d, const LaunchCfg& c, int optin, bool primal, bool tune);
 // threads of a block of these kernels at most, for the element size and values per thread
 inline int band_threads_max(int elem, int vals) { return elem == 8 && vals == 16 ? 256 : 512; }
 // Fills the fast_* part of c for the tiles of d (col_width, upd_rows) and the equation's halo H;

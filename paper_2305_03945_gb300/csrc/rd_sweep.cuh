@@ -1000,7 +1000,7 @@ static cudaError_t launch_iter_k(const Desc& d, State* st, const LaunchCfg& c, c
     if (ev && e == cudaSuccess) e = cudaEventRecordWithFlags(ev[i], s, flags);
   };
   mark(0);
-  if constexpr (PC) {
+  if constexpr (PC && sizeof(T) == 8) {  // (the preconditioner alone is applied in FP64)
     if (c.transform && c.fast_row) {
       if (e == cudaSuccess) e = launch_rowfwd<T>(d, c, s);
       mark(1);
