@@ -764,8 +764,7 @@ void share_tiles(rd_pdhg* h, const Desc& d) {
 // k_primal: two-row bands (one line of 8192 points fills a block), the widest columns that fit up to
 // 32 bytes.  False where they cannot run it.
 template <class T>
-bool plan_long(int nx, int ny, int nc, int H, bool neumann, Desc& d, LaunchCfg& c) {
-  (void)neumann;
+bool plan_long(int nx, int ny, int nc, int H, Desc& d, LaunchCfg& c) {
   Desc p = d;
   LaunchCfg q{};
   q.transform = 1;
@@ -987,7 +986,7 @@ rd_status create_impl(rd_pdhg* h, const rd_grid* grid, rd_bc bc, rd_operator op,
   std::string why;
   Desc d64 = base, d32 = base;
   if (long2d && h->dc && transform && h->opts.fused_update &&
-      plan_long<float>(h->nx, h->ny, h->nc, H, bc == RD_BC_NEUMANN, d32, h->cfg32)) {
+      plan_long<float>(h->nx, h->ny, h->nc, H, d32, h->cfg32)) {
     h->nd3 = 0;
     share_plan(d32, d64);
   } else if (h->nd3) {

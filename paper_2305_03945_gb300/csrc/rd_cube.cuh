@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(BandThreads<T, V>::value) k3_axis(const __grid
                                                                     int nl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
-  if (st && !sweep_active(st, nullptr)) return;  // st = nullptr: the preconditioner alone
+  if (!sweep_active(st, nullptr)) return;
   axis3_body<T, AX, MODE, LOGN, V>(d, nl, blockIdx.x, smem_raw, [] { __syncthreads(); });
 }
 

@@ -26,8 +26,8 @@ namespace rd {
 template <int LOGN, int V>
 struct Rf {
   static_assert(LOGN >= 4 && LOGN <= 13, "lines of 16 .. 8192 points");
-  static_assert(V == 4 || V == 8 || V == 16, "values per thread");
-  static constexpr int LV = V == 16 ? 4 : (V == 8 ? 3 : 2);
+  static_assert(V == 4 || V == 16, "values per thread");
+  static constexpr int LV = V == 16 ? 4 : 2;
   static constexpr int N = 1 << LOGN;
   static constexpr int TPL = N / V;  // threads per line
   static constexpr int P = 1 + (LOGN - (LV - 1) + LV - 1) / LV;
@@ -48,7 +48,7 @@ struct Rf {
 //   rows (lanes along the line), FP32, N >= 256: 8 k_1 + (k_1 >> 1) is distinct modulo 16 over the
 //   16 values of k_1 and differs by 8 within a pair; FP64 and short lines: k_1;
 //   columns (lanes along adjacent lines first, COLS): k_1, an odd stride.
-// V < 16: p + p / 16 + p / 64 (at most 4 lanes on a bank).
+// V = 4: p + p / 16 + p / 64 (at most 4 lanes on a bank).
 template <class T, int LOGN, int V, bool COLS>
 struct Lay {
   using F = Rf<LOGN, V>;
@@ -60,7 +60,7 @@ struct Lay {
   }
   // stored position of natural position p
   static __host__ __device__ __forceinline__ constexpr int at(int p) {
-    if constexpr (V < 16) return p + (p >> 4) + (p >> 6);
+    if constexpr (V == 4) return p + (p >> 4) + (p >> 6);
     else if constexpr (F::P < 4) return p + skew1(p >> F::ll(1));
     else return p + skew1(p >> F::ll(1)) + skew2((p >> F::ll(2)) & (R2 - 1));
   }

@@ -62,14 +62,14 @@ int halo_of(int key) { return key == KK_CH_IMPL || key == KK_CH_SPLIT || key == 
 
 int small_mode(int nx, int ny, int nc, int key, bool neumann, int usable) {
   if (nx >= 2 * kClusterCtas && ny >= 2 * kClusterCtas && nc * nx * ny <= 16384 &&
-      cluster_smem_bytes(nx, ny, nc, halo_of(key), neumann) <= usable)
+      cluster_smem_bytes(nx, ny, nc, halo_of(key)) <= usable)
     return 2;
   if (nx >= 2 && ny >= 2 && nc * nx * ny <= 4096 && small_smem_bytes(nx, ny, nc, neumann) <= usable) return 1;
   return 0;
 }
 
 int small_smem_of(int mode, int nx, int ny, int nc, int key, bool neumann) {
-  return mode == 2 ? cluster_smem_bytes(nx, ny, nc, halo_of(key), neumann) : small_smem_bytes(nx, ny, nc, neumann);
+  return mode == 2 ? cluster_smem_bytes(nx, ny, nc, halo_of(key)) : small_smem_bytes(nx, ny, nc, neumann);
 }
 
 cudaError_t launch_small(const Desc& d, State* st, int mode, cudaStream_t s) {

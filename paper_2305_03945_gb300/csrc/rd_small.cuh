@@ -322,8 +322,7 @@ __host__ __device__ inline int cluster_lines(int lines, int n) {
   return (lines * tpl + 31) / 32 * 32 / tpl;
 }
 
-__host__ __device__ inline int cluster_smem_bytes(int nx, int ny, int nc, int H, bool neumann) {
-  (void)neumann;
+__host__ __device__ inline int cluster_smem_bytes(int nx, int ny, int nc, int H) {
   const int R = ny / kClusterCtas, C = nx / kClusterCtas;
   int b = 0;
   b += 2 * up16(nc * (R + 2 * H) * nx * 4);  // d, u with H halo rows
