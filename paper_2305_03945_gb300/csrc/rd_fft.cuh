@@ -79,7 +79,11 @@ __device__ __forceinline__ void line_sync(int line) {
   else asm volatile("bar.sync %0, %1;" ::"r"(line + 1), "n"(TPL) : "memory");
 }
 
-// w^1 .. w^{R-1} of one job from the table entries w^1, w^2, w^4, w^8 (global table, cached).
+// w^1 .. w^{R-1} of one job from a few table entries (global table, cached), with no more rounding than in the
+// radix-8 passes of rd_device.cuh, whose twiddles are products of three entries at most.  Radix 16: w^1, w^2, w^8 and
+// w^13 are read, and every other power is the product of two of them, or of one and another's conjugate.  (Products
+// of up to four of w^1, w^2, w^4, w^8 raised the rounding floor of the FP32 inner solves: 8192^2, error of a step
+// against 64 bits 7.1e-12 -> 8.4e-12.)
 template <class T, int R>
 __device__ __forceinline__ void rf_twiddles(const cx<T>* __restrict__ tw, int step, cx<T>* w) {
   w[1] = ldg(tw + step);
@@ -87,16 +91,25 @@ __device__ __forceinline__ void rf_twiddles(const cx<T>* __restrict__ tw, int st
     w[2] = ldg(tw + 2 * step);
     w[3] = cmul(w[1], w[2]);
   }
-  if constexpr (R > 4) {
+  if constexpr (R == 8) {
     w[4] = ldg(tw + 4 * step);
     w[5] = cmul(w[1], w[4]);
     w[6] = cmul(w[2], w[4]);
     w[7] = cmul(w[3], w[4]);
   }
-  if constexpr (R > 8) {
+  if constexpr (R == 16) {
     w[8] = ldg(tw + 8 * step);
-#pragma unroll
-    for (int r = 9; r < 16; ++r) w[r] = cmul(w[r - 8], w[8]);
+    w[13] = ldg(tw + 13 * step);  // (step < N / 16)
+    w[4] = cmul(w[2], w[2]);
+    w[5] = cmul_tw<T, 1>(w[13], w[8]);  // w^13 conj(w^8), ...
+    w[6] = cmul_tw<T, 1>(w[8], w[2]);
+    w[7] = cmul_tw<T, 1>(w[8], w[1]);
+    w[9] = cmul(w[1], w[8]);
+    w[10] = cmul(w[2], w[8]);
+    w[11] = cmul_tw<T, 1>(w[13], w[2]);
+    w[12] = cmul_tw<T, 1>(w[13], w[1]);
+    w[14] = cmul(w[1], w[13]);
+    w[15] = cmul(w[2], w[13]);
   }
 }
 
