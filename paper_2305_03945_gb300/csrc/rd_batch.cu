@@ -35,6 +35,7 @@
 #include "rd_batch_lines.h"
 #include "rd_launch3.h"
 #include "rd_launch_small.h"
+#include "rd_mu.h"
 
 namespace rd {
 
@@ -404,6 +405,7 @@ struct rd_batch {
   // pi k / (2 kBatchMaxSide) for the eigenvalues
   cx<float>* d_tables = nullptr;
   std::vector<double> sines;
+  std::vector<long double> sines_l;
   std::vector<SlotHost> slots;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -450,6 +452,7 @@ rd_status make_tables(rd_batch* b) {
   const long double pi = 3.141592653589793238462643383279502884L;
   constexpr int N = kBatchMaxSide;
   b->sines.resize(2 * N + 1);
+  b->sines_l.resize(2 * N + 1);
   std::vector<cx<float>> tab(2 * (2 * N - 4));
   std::vector<cx<float>> tw(N), dc(N);
   for (int k = 0; k < N; ++k) {
@@ -458,7 +461,10 @@ rd_status make_tables(rd_batch* b) {
     const long double q = pi * k / (2.0L * N);
     dc[k] = cx<float>{(float)cosl(q), (float)sinl(q)};
   }
-  for (int k = 0; k <= 2 * N; ++k) b->sines[k] = (double)sinl(pi * k / (2.0L * N));
+  for (int k = 0; k <= 2 * N; ++k) {
+    b->sines_l[k] = sinl(pi * k / (2.0L * N));
+    b->sines[k] = (double)b->sines_l[k];
+  }
   for (int n = 4; n <= N; n *= 2)
     for (int k = 0; k < n; ++k) {
       tab[n - 4 + k] = tw[k * (N / n)];
@@ -476,8 +482,8 @@ const cx<float>* rotations_of(const rd_batch* b, int n) { return b->d_tables + (
 void append_mu(const rd_batch* b, int n, bool neumann, double h, std::vector<float>& mu) {
   const int step = (neumann ? 1 : 2) * (kBatchMaxSide / n);
   for (int k = 0; k < n; ++k) {
-    const double sn = b->sines[k * step];
-    mu.push_back((float)(4.0 / (h * h) * sn * sn));
+    const int q = k * step;
+    mu.push_back(eigenvalue32(b->sines[q], b->sines_l[q], h));
   }
 }
 

@@ -120,6 +120,13 @@ static size_t names_out(const std::vector<std::string>& v, char* out, size_t cap
 }
 size_t fake_launched(char* out, size_t cap) { return names_out(g_launched, out, cap); }
 size_t fake_limits(char* out, size_t cap) { return names_out(g_attr, out, cap); }
+// whether some device allocation holds these bytes
+int fake_contains(const void* bytes, size_t n) {
+  Lock lk(g_mu);
+  for (auto& [p, len] : g_allocs)
+    if (memmem(p, len, bytes, n)) return 1;
+  return 0;
+}
 int fake_outer_after_inner(int inner) { return rd::outer_after_inner(inner); }
 // The plan of k_primal for bands of `rows` rows: whether it runs, and its shared memory.
 int fake_plan_band(int elem, int nx, int ny, int nc, int H, int rows, int limit, int* smem_primal) {

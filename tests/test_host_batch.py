@@ -66,3 +66,23 @@ with rd.Batch(1 << 28, 4, stream=0) as b:
     assert lib.fake_alloc_calls() == n
     lib.fake_refuse_alloc(0)
 """)
+
+
+@pytest.mark.parametrize("length", [6.58562070071191, 0.9680646812275848, 5.784860330543764, 1.0])
+def test_eigenvalues_are_rounded_once(lib, length):
+    """The FP32 eigenvalues of a slot are the long double ones rounded: on the first three lengths, rounding them to
+    double on the way changes one of them."""
+    F.run(lib, SERVE + """
+import ctypes
+L = np.longdouble
+length, n = %r, 1024
+lib.fake_slots(1)
+with rd.Batch(1 << 25, 1, stream=0) as b:
+    pb, u0 = request(1, (16, n))
+    serve(b, [(pb.replace(lx=length), u0)])
+    h = L(length / n)
+    sn = np.sin(L("3.141592653589793238462643383279502884") * np.arange(n).astype(L) / L(2 * n))
+    mu = (L(4) / (h * h) * sn * sn).astype(np.float32)
+    lib.fake_contains.argtypes = [ctypes.c_void_p, ctypes.c_size_t]
+    assert lib.fake_contains(mu.ctypes.data, mu.nbytes) == 1
+""" % length)
