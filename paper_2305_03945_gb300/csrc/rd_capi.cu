@@ -87,8 +87,11 @@ bool use_pingpong(int fft_buffers, int threads, int smem_inplace, int smem_pp) {
 // Column width of k_fcol (sides of 16 points and more): 32-byte row segments, wider while a block has
 // less than a warp, narrower where a block does not hold that many lines.  Measured in FP32 (column
 // kernel): 2048^2 x 2 16-byte segments 67 us, 32-byte 55 us, 64-byte (one block per SM) 108 us;
-// 1024^2 16.5, 14.1, 16.2 us; 512^2 and 1024 x 128 are flat from 16 to 64 bytes.  Lines too long or
-// too short for it: `old`, the width planned for k_col.
+// 1024^2 16.5, 14.1, 16.2 us; 512^2 and 1024 x 128 are flat from 16 to 64 bytes.  FP64 is bound by an SM's
+// narrow pipes, so its columns spread over twice the SMs, a warp or more each, where half the chip would idle
+// (steps with 16-byte / 32-byte segments, grids of 16 and 256 by 1024-point columns 1.69 / 2.41 and 2.56 / 3.26 ms; of 16
+// and 256 by 512-point ones 1.30 / 1.61 and 1.63 / 1.94 ms; 256^2 1.47 / 1.50 ms; more blocks than SMs, 512^2: equal).
+// Lines too long or too short for it: `old`, the width planned for k_col.
 template <class T>
 int plan_col_width(int nx, int old, Desc d, LaunchCfg c) {
   int C = std::min(nx, 32 / (int)sizeof(T));
@@ -100,6 +103,7 @@ int plan_col_width(int nx, int old, Desc d, LaunchCfg c) {
   if (plan(C))
     while (c.thr_fcol < 32 && C < nx && plan(2 * C)) C *= 2;
   while (C > 2 && !plan(C)) C /= 2;
+  while (sizeof(T) == 8 && C > 2 && plan(C) && c.thr_fcol >= 64 && 2 * d.ncomp * (nx / C) <= kTargetBlocks) C /= 2;
   return plan(C) ? C : old;
 }
 

@@ -32,3 +32,15 @@ def test_column_widths_are_timed_on_the_kernel_that_runs(lib, ny, threads, tma, 
     assert out[-2] == runs, out
     if runs == "tma":  # (a tile of less than 16-byte rows has no tensor map)
         assert int(out[-1]) >= 4
+
+
+@pytest.mark.parametrize("nx,ny,width", [(16, 1024, 2), (64, 512, 2), (256, 1024, 2), (512, 512, 4), (1024, 1024, 4), (16, 64, 4)])
+def test_fp64_columns_spread_over_the_chip(lib, nx, ny, width):
+    """Pairs of columns while twice the blocks still fit one wave and a block keeps a warp; else 32-byte segments."""
+    out = F.run(lib, """
+from paper_2305_03945_gb300 import workloads as WL
+pb = WL.Problem(nx=%d, ny=%d, lx=1.0, ly=1.0, bc="neumann", op="laplacian", kind="allen_cahn", dt=1e-3, a=0.05, b=20.0,
+                tol=1e-11, tol_kind="f_rel")
+print("WIDTH", rd.Solver(pb, stream=0).stats()["plan_col_width"])
+""" % (nx, ny)).split()
+    assert out[-2:] == ["WIDTH", str(width)], out
