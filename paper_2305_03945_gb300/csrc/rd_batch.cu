@@ -562,7 +562,9 @@ void launch_branch(rd_batch* b, int g, int part, cudaStream_t s) {
 // branch of its own through all its iterations, so that the kernels of one fill the launch gaps and
 // idle SMs of the others (one chain through all of them: 28 launches in a row per iteration of a mix
 // of two kinds with cubes).  An iteration of the one-launch slots is a whole inner solve, as long as
-// several sweeps: their branch has a quarter of the iterations, so that no branch waits long for it.
+// several sweeps: their branch has a quarter of the iterations, so that no branch waits long for it, or
+// half where no other kind of branch is there to wait (16 runs of 5 steps, a quarter / half / all: 4 x 4 3.0 / 2.1 /
+// 2.4 ms, 64 x 64 3.8 / 3.6 / 3.6 ms; of one step: 64 x 64 1.51 / 1.57 / 1.68 ms).
 rd_status rebuild_graph(rd_batch* b) {
   if (b->gexec) {
     cudaGraphExecDestroy(b->gexec);
@@ -574,9 +576,11 @@ rd_status rebuild_graph(rd_batch* b) {
   }
   cudaError_t e = cudaSuccess;
   std::vector<int> live;
+  bool only_small = true;
   for (int k = 0; k < kBatchParts * kBatchGroups; ++k) {
     if (part_items(b, k / kBatchParts, k % kBatchParts) == 0) continue;
     live.push_back(k);
+    only_small = only_small && k % kBatchParts == 1;
     if (!b->branch_stream[k]) e = cudaStreamCreateWithFlags(&b->branch_stream[k], cudaStreamNonBlocking);
     if (e == cudaSuccess && !b->ev_join[k]) e = cudaEventCreateWithFlags(&b->ev_join[k], cudaEventDisableTiming);
     if (e != cudaSuccess) return bfail(RD_ERR_CUDA, std::string("batch branches: ") + cudaGetErrorString(e));
@@ -588,7 +592,7 @@ rd_status rebuild_graph(rd_batch* b) {
     const int part = k % kBatchParts;
     cudaStream_t s = b->branch_stream[k];
     cudaStreamWaitEvent(s, b->ev_fork, 0);
-    const int iters = part == 1 ? std::max(1, b->opts.graph_k / 4) : b->opts.graph_k;
+    const int iters = part == 1 ? std::max(1, b->opts.graph_k / (only_small ? 2 : 4)) : b->opts.graph_k;
     for (int i = 0; i < iters; ++i) launch_branch(b, k / kBatchParts, part, s);
     cudaEventRecord(b->ev_join[k], s);
     cudaStreamWaitEvent(b->cap_stream, b->ev_join[k], 0);

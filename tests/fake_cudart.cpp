@@ -30,6 +30,7 @@ std::vector<std::string> g_attr;               // kernels whose shared-memory li
 std::map<std::string, float> g_cost;           // part of a kernel's name -> time of a launch
 std::map<void*, size_t> g_events;              // event -> launches when it was recorded
 bool g_refuse_alloc = false;
+bool g_hold = false;                           // graphs leave the slots as they are
 long g_alloc_calls = 0;                        // cudaMalloc and cudaFree
 size_t g_slots = 0;                            // slots of the batch under test
 int g_state_status[2] = {rd::ST_CONVERGED, rd::ST_CONVERGED};
@@ -47,7 +48,7 @@ void run_pending() {
 void finish_graph() {
   Lock lk(g_mu);
   for (auto& [p, n] : g_allocs) {
-    if (g_slots && n == g_slots * sizeof(rd::Slot)) {
+    if (g_slots && !g_hold && n == g_slots * sizeof(rd::Slot)) {
       for (size_t k = 0; k < g_slots; ++k) {
         rd::Slot& s = reinterpret_cast<rd::Slot*>(p)[k];
         if (s.phase != rd::PH_BEGIN) continue;
@@ -107,6 +108,10 @@ extern "C" {
 
 // --- what the tests set and read ---
 void fake_refuse_alloc(int on) { g_refuse_alloc = on; }
+void fake_hold(int on) {
+  Lock lk(g_mu);
+  g_hold = on;
+}
 long fake_alloc_calls() { return g_alloc_calls; }
 void fake_slots(size_t n) { g_slots = n; }
 void fake_status(int outer, int inner) { g_state_status[0] = outer, g_state_status[1] = inner; }

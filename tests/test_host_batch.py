@@ -86,3 +86,26 @@ with rd.Batch(1 << 25, 1, stream=0) as b:
     lib.fake_contains.argtypes = [ctypes.c_void_p, ctypes.c_size_t]
     assert lib.fake_contains(mu.ctypes.data, mu.nbytes) == 1
 """ % length)
+
+
+def test_small_solves_alone_fill_a_longer_graph(lib):
+    """Inner solves per graph of the one-launch slots: half of graph_k alone, a quarter beside other branches."""
+    F.run(lib, SERVE + """
+lib.fake_slots(4)
+def solves():
+    return sum("k_small" in n for n in F.names(lib.fake_launched))
+with rd.Batch(1 << 26, 4, graph_k=16, stream=0) as b:
+    serve(b, [request(0, (4, 4))])
+    assert solves() == 8, solves()
+with rd.Batch(1 << 26, 4, graph_k=16, stream=0) as b:
+    n, ids = solves(), []
+    lib.fake_hold(1)
+    for k, s in enumerate([(256, 256), (4, 4)]):  # the second joins the first, still running
+        ids.append(b.submit(*request(k, s), 1))
+        t0 = time.time()
+        while b.stats()["admitted"] < k + 1 and time.time() - t0 < 30:
+            time.sleep(0.01)
+    lib.fake_hold(0)
+    assert len(drain(b, ids)) == 2
+    assert solves() - n == 4, solves() - n
+""")
