@@ -324,7 +324,9 @@ class Solver:
 class Batch:
     """Continuous-batching server of implicit-step runs (rd_batch_*).  Requests are
     ``workloads.Problem`` records plus a host float64 initial state and a step count; results
-    come back through ``poll``, final states in the host arrays returned by ``submit``."""
+    come back through ``poll``, final states in the host arrays returned by ``submit``.
+    ``autotune`` is accepted and has no effect: the batched kernels' launch shapes follow from the
+    grids, there is nothing to measure."""
 
     def __init__(self, hbm_budget_bytes, max_slots, graph_k=8, max_iter=10000, dc_inner_rtol=None,
                  dc_max_outer=None, stream=None, small_solve=1, autotune=1):
