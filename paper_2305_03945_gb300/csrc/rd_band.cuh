@@ -167,7 +167,7 @@ __device__ __forceinline__ void fcol_body(const Desc& d, int blk, unsigned char*
 template <class T, int V>
 struct BandThreads { static constexpr int value = sizeof(T) == 8 && V == 16 ? 256 : 512; };
 // of k_fcol: FP32 lines of 4096 and 8192 points take 1024 threads to hold two lines or more; at 64
-// registers these and the 2048-point ones spill 150 to 210 bytes (k_fcol_tma 50 to 110)
+// registers these and the 2048-point ones spill 160 to 240 bytes (k_fcol_tma 50 to 130)
 template <class T, int LOGN, int V>
 struct ColThreads {
   static constexpr int value = LOGN >= 12 && sizeof(T) == 4 ? 1024 : BandThreads<T, V>::value;
@@ -572,11 +572,17 @@ __host__ __device__ inline int primal_smem_bytes(int nc, int rows, int H, int nx
 }
 
 // Threads of a k_primal block at most, and the blocks an SM shall hold (the register cap).  FP32 lines of
-// 2048 points and more: 1024 threads, 64 registers (two species spill 100 bytes): two blocks of four rows
-// or one of eight per SM; FP32 five-point kinds at V = 16 on shorter lines: two blocks of 512.
+// 2048 points and more: 1024 threads, 64 registers (two species spill 20 to 40 bytes): two blocks of four rows
+// or one of eight per SM; but 512 threads at 128 registers for Cahn-Hilliard, whose thirteen-point stencils of d and
+// u spill 240 to 380 bytes at 64 (steps at 64 / 128 registers: split 2048^2 6.20 / 5.36 ms, 4096^2 22.3 / 21.2 ms, 256 x 4096
+// 2.44 / 2.40 ms; implicit 2048^2 5.97 / 5.13 ms; the biharmonic alone, which does not spill, 3.85 / 4.01 ms).  FP32
+// five-point kinds at V = 16 on shorter lines: two blocks of 512.  (primal_wide: the same rule for the planner.)
+inline bool primal_wide(const Desc& d, int H, int elem, int vals) {
+  return elem == 4 && vals == 16 && d.nx >= 2048 && !(H == 2 && d.kind != RX_NONE);
+}
 template <class T, int K, int LOGN, int V>
 struct PrimalBlock {
-  static constexpr bool wide = sizeof(T) == 4 && V == 16 && LOGN >= 11;
+  static constexpr bool wide = sizeof(T) == 4 && V == 16 && LOGN >= 11 && !(KT<K>::biharm && KT<K>::nonlinear);
   static constexpr int threads = wide ? 1024 : BandThreads<T, V>::value;
   static constexpr int blocks = sizeof(T) == 4 && V == 16 && !wide && !KT<K>::biharm ? 2 : 1;
 };

@@ -191,7 +191,7 @@ void plan_band(const Desc& d, int H, int smem_limit, LaunchCfg& c) {
   }
   if (has_len<T>(d.lognx, c.vrow)) {
     const int tpl = d.nx / c.vrow, len = line_len<T, false>(d.lognx, c.vrow);
-    const int cap = d.nx >= 2048 && sizeof(T) == 4 && c.vrow == 16 ? 1024 : band_threads_max(sizeof(T), c.vrow);  // k_primal
+    const int cap = primal_wide(d, H, sizeof(T), c.vrow) ? 1024 : band_threads_max(sizeof(T), c.vrow);  // k_primal
     // k_dual: blocks of one warp or one line at least, of up to 256 threads once the lines give
     // two blocks per SM
     const int lines = nc * (d.ny / 2);
